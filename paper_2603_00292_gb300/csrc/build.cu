@@ -22,269 +22,400 @@
 namespace grt {
 
 // ======================================================================= radix sort
+// Stable least-significant-digit radix sort of (key, value) pairs, 8 bits a pass, one
+// launch a pass (Adinolfi and Merrill's single-pass sort, "Onesweep", 2022, over Merrill
+// and Garland's decoupled look-back, 2016). The digit histograms of every pass depend on
+// the keys alone and are counted once, before the first pass; a pass then takes its tiles
+// in order from a ticket, ranks a tile's keys on chip, learns from the tiles before it how
+// many of each digit they hold, and writes its own in digit order.
+//
+// What bounds it: a pass moves 2 x 12 B (8 B with 32-bit keys) a pair, which L2 holds at
+// every size that fits it, so the time is the chain load -> rank -> look back -> store of
+// one wave of tiles, all of which run at once, and the instructions of ranking. The
+// look-back is therefore two levels deep: tiles add their counts to their group's, a tile
+// sums the groups before its own and the tiles before it in its group, and a group's first
+// tile publishes what lies before the group. Measured on a 1.23 M build with 63-bit codes (8
+// passes): groups of 8, 472-478 us; one level 491; groups of 16, 495-511. A pass takes 16 us
+// there and 6 at 131,072 32-bit keys. The form before it (a histogram launch, a scan of 256
+// counters per block on ONE block, a scatter straight from registers) took 88 us, 55 of them
+// in the scan, and 21 us. Tiles of 2,048 keys at four blocks per SM (64 registers): the 603
+// tiles of 1.23 M keys run in one wave (tiles of 3,072: 486 us, of 1,024: 509).
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 16;
+constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kRadix = 256;
-constexpr int kMaxSortBlocks = 1024;
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 8;
+constexpr int kMaxPasses = 8;
+static_assert(kSortThreads == kRadix, "one thread per digit");
+// Look-back words, 64 bits each so that a count up to 2^32 and its state are one store: a
+// tile's count of a digit with bit 32 set once it is there; a group's count with the number
+// of its tiles that have added theirs above it; the count before a group with bit 32 set.
+constexpr unsigned long long kLookOne = 1ull << 32;
+constexpr uint32_t kLookGroup = 8;          // tiles of a group
+constexpr int kLookWindow = 2;              // groups read at a time
+constexpr uint32_t kLookSpins = 1u << 22;   // polls of one word, far above any tile's time
 
-size_t sortScratchBytes(uint32_t) { return (size_t)kRadix * kMaxSortBlocks * sizeof(uint32_t); }
-
-struct SortGrid {
-    unsigned tiles, tilesPerBlock, blocks;
+// Scratch of a sort: digit counts of every pass, the passes' tile tickets, and two sets of
+// look-back words used in turn (a pass clears the next one's). A set: the tiles' words, then
+// the groups' counts, then the counts before the groups, kRadix words each.
+struct SortScratch {
+    uint32_t* hist;             // kMaxPasses x kRadix
+    uint32_t* tickets;          // kMaxPasses
+    unsigned long long* look[2];
 };
-
-static SortGrid sortGrid(uint32_t n, int sms) {
-    SortGrid g;
-    g.tiles = std::max(1u, ceilDiv(n, kSortTile));
-    unsigned want = std::min<unsigned>(g.tiles, std::min<unsigned>(kMaxSortBlocks, (unsigned)std::max(1, sms) * 2));
-    g.tilesPerBlock = ceilDiv(g.tiles, want);
-    g.blocks = ceilDiv(g.tiles, g.tilesPerBlock);
-    return g;
+constexpr size_t kSortHeadBytes = (size_t)kMaxPasses * kRadix * 4 + 256;
+__host__ __device__ inline uint32_t lookGroups(uint32_t tiles) { return (tiles + kLookGroup - 1) / kLookGroup; }
+static size_t lookBytes(uint32_t n) {
+    const uint32_t tiles = std::max(1u, ceilDiv(n, kSortTile));
+    return ((size_t)tiles + 2 * (size_t)lookGroups(tiles)) * kRadix * sizeof(unsigned long long);
+}
+size_t sortScratchBytes(uint32_t n) { return kSortHeadBytes + 2 * lookBytes(n); }
+static SortScratch sortScratch(void* p, uint32_t n) {
+    char* c = static_cast<char*>(p);
+    SortScratch S;
+    S.hist = reinterpret_cast<uint32_t*>(c);
+    S.tickets = S.hist + kMaxPasses * kRadix;
+    S.look[0] = reinterpret_cast<unsigned long long*>(c + kSortHeadBytes);
+    S.look[1] = reinterpret_cast<unsigned long long*>(c + kSortHeadBytes + lookBytes(n));
+    return S;
 }
 
+__device__ __forceinline__ unsigned long long loadRelaxed(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void storeRelaxed(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Word *p, already read as w, once it has reached `ready`. The tile that brings it there
+// started before this one, so it always gets there; the limit only ends a wait on a
+// corrupted word, and the pass's stores are bounded all the same.
+__device__ __forceinline__ uint32_t lookValue(const unsigned long long* p, unsigned long long w,
+                                              unsigned long long ready, uint32_t* error) {
+    for (uint32_t spin = 0; w < ready; ++spin) {
+        if (spin == kLookSpins) {
+            latchError(error, GRT_ERROR_TIMEOUT);
+            break;
+        }
+        w = loadRelaxed(p);
+    }
+    return (uint32_t)w;
+}
+
+// Adds key k's digits to the block's histograms h[pass][digit]. A warp whose lanes share a
+// digit (the high digits of neighbouring primitives) adds them at once: 32 atomics on one
+// word of shared memory would run one after another.
 template <typename K>
-__global__ void __launch_bounds__(kSortThreads) sortUpsweep(const K* __restrict__ keys, uint32_t n, int shift,
-                                                            uint32_t tilesPerBlock, uint32_t* __restrict__ counts,
-                                                            uint32_t blocks) {
-    __shared__ uint32_t h[kSortWarps][kRadix];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    for (int d = tid; d < kSortWarps * kRadix; d += kSortThreads) (&h[0][0])[d] = 0;
-    __syncthreads();
-    const size_t begin = (size_t)blockIdx.x * tilesPerBlock * kSortTile;
-    const size_t end = min((size_t)n, begin + (size_t)tilesPerBlock * kSortTile);
-    for (size_t i = begin + tid; i < end; i += kSortThreads) {
-        const uint32_t d = (uint32_t)(keys[i] >> shift) & (kRadix - 1);
-        atomicAdd(&h[warp][d], 1u);
-    }
-    __syncthreads();
-    for (int d = tid; d < kRadix; d += kSortThreads) {
-        uint32_t s = 0;
-#pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) s += h[w][d];
-        counts[(size_t)d * blocks + blockIdx.x] = s;
+__device__ __forceinline__ void countDigits(K k, bool valid, int passes, uint32_t (*h)[kRadix]) {
+    const unsigned act = __ballot_sync(0xffffffffu, valid);
+    if (!act) return;
+    const int leader = __ffs(act) - 1;
+    for (int p = 0; p < passes; ++p) {
+        const uint32_t d = (uint32_t)(k >> (8 * p)) & (kRadix - 1);
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d, leader);
+        if (__all_sync(0xffffffffu, !valid || d == d0)) {
+            if ((int)(threadIdx.x & 31u) == leader) atomicAdd(&h[p][d0], (uint32_t)__popc(act));
+        } else if (valid) {
+            atomicAdd(&h[p][d], 1u);
+        }
     }
 }
 
-// Exclusive prefix sum in place over `total` counters (one block).
-__global__ void __launch_bounds__(kScanThreads) sortScan(uint32_t* __restrict__ counts, uint32_t total) {
-    __shared__ uint32_t warpSums[kScanThreads / 32];
-    __shared__ uint32_t carryS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) carryS = 0;
-    __syncthreads();
-    for (uint32_t base = 0; base < total; base += kScanThreads * kScanItems) {
-        uint32_t v[kScanItems];
-        uint32_t sum = 0;
-        const uint32_t my = base + (uint32_t)tid * kScanItems;
-#pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            v[i] = (my + i < total) ? counts[my + i] : 0u;
-            sum += v[i];
-        }
-        uint32_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) warpSums[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = warpSums[lane];
-            uint32_t wi = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-                if (lane >= o) wi += t;
-            }
-            warpSums[lane] = wi - w;  // exclusive
-        }
-        __syncthreads();
-        uint32_t run = carryS + warpSums[warp] + (incl - sum);
-#pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            if (my + i < total) counts[my + i] = run;
-            run += v[i];
-        }
-        __syncthreads();
-        if (tid == kScanThreads - 1) carryS = run;
-        __syncthreads();
+__device__ __forceinline__ void flushDigits(int passes, const uint32_t (*h)[kRadix], uint32_t* hist) {
+    for (int j = threadIdx.x; j < passes * kRadix; j += blockDim.x) {
+        const uint32_t c = (&h[0][0])[j];
+        if (c) atomicAdd(hist + j, c);
     }
 }
 
-// Up to kFusedScanBlocks blocks the downsweep derives its digit offsets from the raw
-// per-block counts itself (every block reads all kRadix x blocks counts from L2), so a
-// radix pass is two launches instead of three; the offsets are those sortScan gives.
-constexpr uint32_t kFusedScanBlocks = 64;
+// Blocks that count digits are large and few (countBlocks: two per SM fill it): each ends in
+// an atomic per nonzero count on the same kMaxPasses x kRadix words. With eight blocks of
+// 256 threads per SM the Morton kernel took 20 us at 1.23 M keys, 10 of them there.
+constexpr int kCountThreads = 1024;
+static unsigned countBlocks(Context* ctx, uint32_t n) {
+    return std::min(ceilDiv(n, kCountThreads), 2u * (unsigned)std::max(1, smCount(ctx)));
+}
 
-template <typename K, bool FUSED = false>
-__global__ void __launch_bounds__(kSortThreads) sortDownsweep(const K* __restrict__ keysIn,
-                                                              const uint32_t* __restrict__ valsIn,
-                                                              K* __restrict__ keysOut, uint32_t* __restrict__ valsOut,
-                                                              uint32_t n, int shift, uint32_t tilesPerBlock,
-                                                              uint32_t tiles, const uint32_t* __restrict__ offsets,
-                                                              uint32_t blocks) {
+// Digit counts of every pass of n keys (hist zeroed).
+template <typename K>
+__global__ void __launch_bounds__(kCountThreads) sortHistogramKernel(const K* __restrict__ keys, uint32_t n, int passes,
+                                                                    uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[kMaxPasses][kRadix];
+    for (int j = threadIdx.x; j < passes * kRadix; j += kCountThreads) (&h[0][0])[j] = 0u;
+    __syncthreads();
+    for (size_t b = (size_t)blockIdx.x * kCountThreads; b < n; b += (size_t)gridDim.x * kCountThreads) {
+        const size_t i = b + threadIdx.x;
+        countDigits<K>(i < n ? keys[i] : (K)0, i < n, passes, h);
+    }
+    __syncthreads();
+    flushDigits(passes, h, hist);
+}
+
+// Exclusive prefix sum of one value per thread over the block (every thread calls it).
+__device__ __forceinline__ uint32_t blockExclusive(uint32_t v, uint32_t* warpSums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) warpSums[warp] = incl;
+    __syncthreads();
+    uint32_t base = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) base += w < warp ? warpSums[w] : 0u;
+    return base + incl - v;
+}
+
+// The lanes (of those with ok) whose low eight bits equal this lane's, one vote per bit: a
+// __match_any_sync in its place made ranking the longest part of a pass (0.8 us a key of a
+// thread). 0 where ok is false.
+__device__ __forceinline__ uint32_t digitPeers(uint32_t d, bool ok) {
+    uint32_t peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (d >> b) & 1u;
+        const uint32_t m = __ballot_sync(0xffffffffu, set);
+        peers &= set ? m : ~m;
+    }
+    return ok ? peers : 0u;
+}
+
+// One radix pass over one tile. IDENTITY: the values are the positions (a first pass that
+// need not read them).
+template <typename K, bool IDENTITY>
+__global__ void __launch_bounds__(kSortThreads, 4) sortPassKernel(const K* __restrict__ keysIn,
+                                                               const uint32_t* __restrict__ valsIn,
+                                                               K* __restrict__ keysOut, uint32_t* __restrict__ valsOut,
+                                                               uint32_t n, int pass, const uint32_t* __restrict__ hist,
+                                                               uint32_t* tickets, unsigned long long* look,
+                                                               unsigned long long* lookNext, uint32_t tiles,
+                                                               uint32_t* error) {
     __shared__ uint32_t warpHist[kSortWarps][kRadix];
-    __shared__ uint32_t digitBase[kRadix];
-    __shared__ uint32_t tileTotal[kRadix];
+    __shared__ uint32_t outBase[kRadix];
+    __shared__ uint32_t sums[2][kSortWarps];
+    __shared__ K sKeys[kSortTile];
+    __shared__ uint32_t sVals[kSortTile];
+    __shared__ uint32_t sTile;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t ltMask = (1u << lane) - 1u;
-    if constexpr (FUSED) {
-        static_assert(kSortThreads == kRadix, "one thread per digit");
-        // offsets[d * blocks + b] are the raw counts: this block's base for digit d is the
-        // sum of all counts of smaller digits plus those of earlier blocks in digit d
-        uint32_t total = 0, before = 0;
-        for (uint32_t b = 0; b < blocks; ++b) {
-            const uint32_t c = offsets[(size_t)tid * blocks + b];
-            total += c;
-            before += b < blockIdx.x ? c : 0u;
-        }
-        uint32_t incl = total;  // exclusive scan of the digit totals over the block
+    const int shift = 8 * pass;
+    if (tid == 0) sTile = atomicAdd(tickets + pass, 1u);  // tiles start in order: a tile only waits for running ones
+    const uint32_t digitTotal = hist[pass * kRadix + tid];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) tileTotal[warp] = incl;
-        __syncthreads();
-        uint32_t warpBase = 0;
-        for (int w = 0; w < warp; ++w) warpBase += tileTotal[w];
-        __syncthreads();
-        digitBase[tid] = warpBase + incl - total + before;
+    for (int w = 0; w < kSortWarps; ++w) warpHist[w][tid] = 0u;
+    __syncthreads();
+    const uint32_t tile = sTile;
+    const uint32_t first = tile * (uint32_t)kSortTile;
+    const uint32_t count = min((uint32_t)kSortTile, n - first);
+    K k[kSortItems];
+    uint32_t v[kSortItems], rank[kSortItems];
 #pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) warpHist[w][tid] = 0;
-    } else {
-        for (int d = tid; d < kRadix; d += kSortThreads) {
-            digitBase[d] = offsets[(size_t)d * blocks + blockIdx.x];
+    for (int i = 0; i < kSortItems; ++i) {
+        const uint32_t j = (uint32_t)(warp * kSortItems + i) * 32u + (uint32_t)lane;
+        const bool ok = j < count;
+        k[i] = ok ? keysIn[(size_t)first + j] : (K)0;
+        v[i] = IDENTITY ? first + j : ok ? valsIn[(size_t)first + j] : 0u;
+    }
+    const uint32_t group = tile / kLookGroup;
+    const size_t groupsAt = (size_t)tiles * kRadix + tid, beforeAt = groupsAt + (size_t)lookGroups(tiles) * kRadix;
+    storeRelaxed(lookNext + (size_t)tile * kRadix + tid, 0ull);
+    if (tile % kLookGroup == 0) {
+        storeRelaxed(lookNext + groupsAt + (size_t)group * kRadix, 0ull);
+        storeRelaxed(lookNext + beforeAt + (size_t)group * kRadix, 0ull);
+    }
+    uint32_t peers[kSortItems];
 #pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) warpHist[w][d] = 0;
-        }
+    for (int i = 0; i < kSortItems; ++i) {
+        const bool ok = (uint32_t)(warp * kSortItems + i) * 32u + (uint32_t)lane < count;
+        peers[i] = digitPeers((uint32_t)(k[i] >> shift), ok);
+    }
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const uint32_t d = (uint32_t)(k[i] >> shift) & (kRadix - 1);
+        const uint32_t b = warpHist[warp][d];
+        __syncwarp();
+        if (lane == __ffs(peers[i]) - 1) warpHist[warp][d] = b + __popc(peers[i]);
+        __syncwarp();
+        rank[i] = b + __popc(peers[i] & ltMask);
     }
     __syncthreads();
-    const unsigned t0 = blockIdx.x * tilesPerBlock;
-    const unsigned t1 = min(tiles, t0 + tilesPerBlock);
-    for (unsigned tile = t0; tile < t1; ++tile) {
-        const size_t base = (size_t)tile * kSortTile + (size_t)warp * 32 * kSortItems;
-        K k[kSortItems];
-        uint32_t v[kSortItems], dg[kSortItems], rank[kSortItems];
+    // thread = digit: the warps' counts become each warp's first position in the tile's run
+    uint32_t total = 0;
 #pragma unroll
-        for (int i = 0; i < kSortItems; ++i) {
-            const size_t idx = base + (size_t)i * 32 + lane;
-            const bool ok = idx < n;
-            k[i] = ok ? keysIn[idx] : (K)0;
-            v[i] = ok ? valsIn[idx] : 0u;
-            dg[i] = ok ? ((uint32_t)(k[i] >> shift) & (kRadix - 1)) : (uint32_t)kRadix;
-        }
-#pragma unroll
-        for (int i = 0; i < kSortItems; ++i) {
-            const uint32_t peers = __match_any_sync(0xffffffffu, dg[i]);
-            const int leader = __ffs(peers) - 1;
-            const bool ok = dg[i] < kRadix;
-            const uint32_t b = ok ? warpHist[warp][dg[i]] : 0u;
-            __syncwarp();
-            if (ok && lane == leader) warpHist[warp][dg[i]] = b + __popc(peers);
-            __syncwarp();
-            rank[i] = b + __popc(peers & ltMask);
-        }
-        __syncthreads();
-        for (int d = tid; d < kRadix; d += kSortThreads) {
-            uint32_t run = 0;
-#pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) {
-                const uint32_t t = warpHist[w][d];
-                warpHist[w][d] = run;
-                run += t;
-            }
-            tileTotal[d] = run;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < kSortItems; ++i) {
-            if (dg[i] < kRadix) {
-                const uint32_t pos = digitBase[dg[i]] + warpHist[warp][dg[i]] + rank[i];
-                keysOut[pos] = k[i];
-                valsOut[pos] = v[i];
-            }
-        }
-        __syncthreads();
-        for (int d = tid; d < kRadix; d += kSortThreads) {
-            digitBase[d] += tileTotal[d];
-#pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) warpHist[w][d] = 0;
-        }
-        __syncthreads();
+    for (int w = 0; w < kSortWarps; ++w) {
+        const uint32_t c = warpHist[w][tid];
+        warpHist[w][tid] = total;
+        total += c;
     }
+    storeRelaxed(look + (size_t)tile * kRadix + tid, kLookOne | total);
+    atomicAdd(look + groupsAt + (size_t)group * kRadix, kLookOne + total);
+    const uint32_t digitFirst = blockExclusive(digitTotal, sums[0]);  // over all keys
+    const uint32_t tileFirst = blockExclusive(total, sums[1]);        // within the tile
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) warpHist[w][tid] += tileFirst;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        if ((uint32_t)(warp * kSortItems + i) * 32u + (uint32_t)lane < count) {
+            const uint32_t j = warpHist[warp][(uint32_t)(k[i] >> shift) & (kRadix - 1)] + rank[i];
+            sKeys[j] = k[i];
+            sVals[j] = v[i];
+        }
+    }
+    // the digit's count over the tiles before this one: those of its group, then whole groups
+    // back to one whose own count of earlier keys is there
+    uint32_t before = 0;
+    {
+        unsigned long long w[kLookGroup - 1];
+        const unsigned long long* p = look + (size_t)group * kLookGroup * kRadix + tid;
+        const uint32_t m = tile % kLookGroup;
+#pragma unroll
+        for (uint32_t j = 0; j + 1 < kLookGroup; ++j) w[j] = j < m ? loadRelaxed(p + (size_t)j * kRadix) : kLookOne;
+        uint32_t inGroup = 0;
+        bool open = group > 0;
+        for (uint32_t g = group; open;) {  // groups g - 1, g - 2, ..
+            unsigned long long c[kLookWindow], e[kLookWindow];
+#pragma unroll
+            for (int j = 0; j < kLookWindow; ++j) {
+                const bool in = (uint32_t)j < g;
+                c[j] = in ? loadRelaxed(look + groupsAt + (size_t)(g - 1 - j) * kRadix) : 0ull;
+                e[j] = in ? loadRelaxed(look + beforeAt + (size_t)(g - 1 - j) * kRadix) : kLookOne;
+            }
+#pragma unroll
+            for (int j = 0; j < kLookWindow; ++j) {
+                if (!open) continue;
+                before += lookValue(look + groupsAt + (size_t)(g - 1 - j) * kRadix, c[j], kLookGroup * kLookOne, error);
+                if ((uint32_t)j + 1 == g) {
+                    open = false;
+                } else if (e[j] >= kLookOne) {
+                    before += (uint32_t)e[j];
+                    open = false;
+                }
+            }
+            g -= min(g, (uint32_t)kLookWindow);
+        }
+        if (m == 0 && group > 0) storeRelaxed(look + beforeAt + (size_t)group * kRadix, kLookOne | before);
+#pragma unroll
+        for (uint32_t j = 0; j + 1 < kLookGroup; ++j)
+            if (j < m) inGroup += lookValue(p + (size_t)j * kRadix, w[j], kLookOne, error);
+        before += inGroup;
+    }
+    outBase[tid] = digitFirst + before - tileFirst;
+    __syncthreads();
+    for (uint32_t j = tid; j < count; j += kSortThreads) {
+        const K key = sKeys[j];
+        const uint32_t pos = outBase[(uint32_t)(key >> shift) & (kRadix - 1)] + j;
+        if (pos < n) {  // always, unless a wait ran out
+            keysOut[pos] = key;
+            valsOut[pos] = sVals[j];
+        }
+    }
+}
+
+// The passes over counted digits (scratch.hist) with zeroed tickets and first look-back array.
+template <typename K>
+static grtError sortPasses(Context* ctx, K* const keys[2], uint32_t* const vals[2], uint32_t n, int passes,
+                           const SortScratch& S, bool identity, cudaStream_t s) {
+    const unsigned tiles = ceilDiv(n, kSortTile);
+    for (int p = 0; p < passes; ++p) {
+        const int a = p & 1, b = a ^ 1;
+        if (p == 0 && identity)
+            sortPassKernel<K, true><<<tiles, kSortThreads, 0, s>>>(keys[a], vals[a], keys[b], vals[b], n, p, S.hist,
+                                                                   S.tickets, S.look[a], S.look[b], tiles,
+                                                                   &workspace(ctx)->error);
+        else
+            sortPassKernel<K, false><<<tiles, kSortThreads, 0, s>>>(keys[a], vals[a], keys[b], vals[b], n, p, S.hist,
+                                                                    S.tickets, S.look[a], S.look[b], tiles,
+                                                                    &workspace(ctx)->error);
+        GRT_LAUNCH_CHECK();
+    }
+    noteLaunches(passes);
+    return GRT_SUCCESS;
 }
 
 template <typename K>
 static grtError radixSortT(Context* ctx, K* keys0, K* keys1, uint32_t* vals0, uint32_t* vals1, uint32_t n,
-                           int significantBits, uint32_t* hist, cudaStream_t s, int* finalBuf) {
-    const SortGrid g = sortGrid(n, smCount(ctx));
+                           int significantBits, void* scratch, cudaStream_t s, int* finalBuf) {
     const int passes = (significantBits + 7) / 8;
-    K* kin = keys0;
-    K* kout = keys1;
-    uint32_t* vin = vals0;
-    uint32_t* vout = vals1;
-    for (int p = 0; p < passes; ++p) {
-        const int shift = 8 * p;
-        sortUpsweep<K><<<g.blocks, kSortThreads, 0, s>>>(kin, n, shift, g.tilesPerBlock, hist, g.blocks);
-        if (g.blocks <= kFusedScanBlocks) {
-            sortDownsweep<K, true><<<g.blocks, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, g.tilesPerBlock,
-                                                                      g.tiles, hist, g.blocks);
-            noteLaunches(2);
-        } else {
-            sortScan<<<1, kScanThreads, 0, s>>>(hist, kRadix * g.blocks);
-            sortDownsweep<K><<<g.blocks, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, g.tilesPerBlock,
-                                                                g.tiles, hist, g.blocks);
-            noteLaunches(3);
-        }
-        GRT_LAUNCH_CHECK();
-        std::swap(kin, kout);
-        std::swap(vin, vout);
-    }
+    const SortScratch S = sortScratch(scratch, n);
+    GRT_CUDA(cudaMemsetAsync(scratch, 0, kSortHeadBytes + lookBytes(n), s));
+    sortHistogramKernel<K><<<countBlocks(ctx, n), kCountThreads, 0, s>>>(keys0, n, passes, S.hist);
+    GRT_LAUNCH_CHECK();
+    noteLaunches(1);
+    K* const keys[2] = {keys0, keys1};
+    uint32_t* const vals[2] = {vals0, vals1};
     *finalBuf = passes & 1;
-    return GRT_SUCCESS;
+    return sortPasses<K>(ctx, keys, vals, n, passes, S, false, s);
 }
 
 grtError radixSort(Context* ctx, void* keys0, void* keys1, uint32_t* vals0, uint32_t* vals1, uint32_t n, int keyBytes,
-                   int significantBits, uint32_t* hist, cudaStream_t s, int* finalBuf) {
+                   int significantBits, void* scratch, cudaStream_t s, int* finalBuf) {
     if (n == 0) {
         *finalBuf = 0;
         return GRT_SUCCESS;
     }
     if (keyBytes == 4)
-        return radixSortT<uint32_t>(ctx, (uint32_t*)keys0, (uint32_t*)keys1, vals0, vals1, n, significantBits, hist, s,
-                                    finalBuf);
+        return radixSortT<uint32_t>(ctx, (uint32_t*)keys0, (uint32_t*)keys1, vals0, vals1, n, significantBits, scratch,
+                                    s, finalBuf);
     return radixSortT<unsigned long long>(ctx, (unsigned long long*)keys0, (unsigned long long*)keys1, vals0, vals1, n,
-                                          significantBits, hist, s, finalBuf);
+                                          significantBits, scratch, s, finalBuf);
 }
 
 // ======================================================================= element kernels (A1-A7)
+// Centroids and their bounds. A few blocks per SM loop over the primitives: each block ends
+// in six atomics on the same words, which queued behind one another with a block per 256
+// primitives.
 __global__ void __launch_bounds__(256) primCentroidKernel(PrimSource S, float4* __restrict__ centroids,
                                                           uint32_t* __restrict__ bounds) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = i < S.count;
-    float3 c = make_float3(0.f, 0.f, 0.f);
-    if (valid) {
+    float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < S.count; i += (size_t)gridDim.x * blockDim.x) {
         float3 v[3];
-        c = boxCentroid(primBox(S, i, v));
+        const float3 c = boxCentroid(primBox(S, (uint32_t)i, v));
         centroids[i] = make_float4(c.x, c.y, c.z, 0.f);
+        mn[0] = fminf(mn[0], c.x), mn[1] = fminf(mn[1], c.y), mn[2] = fminf(mn[2], c.z);
+        mx[0] = fmaxf(mx[0], c.x), mx[1] = fmaxf(mx[1], c.y), mx[2] = fmaxf(mx[2], c.z);
     }
-    reduceBounds(c, valid, bounds);
+    reduceBoxBounds(mn, mx, bounds);
 }
 
+// Morton codes, and the digit counts of every radix pass over them (hist zeroed). The
+// values of the pairs are the positions, which the first pass makes itself.
 template <typename K, int BITS>
-__global__ void __launch_bounds__(256) mortonKernel(const float4* __restrict__ centroids, uint32_t n,
-                                                    const uint32_t* __restrict__ bounds, K* __restrict__ keys,
-                                                    uint32_t* __restrict__ vals) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    keys[i] = mortonCode<K, BITS>(centroids[i], bounds);
-    vals[i] = i;
+__global__ void __launch_bounds__(kCountThreads) mortonKernel(const float4* __restrict__ centroids, uint32_t n,
+                                                             const uint32_t* __restrict__ bounds, K* __restrict__ keys,
+                                                             uint32_t* __restrict__ hist) {
+    constexpr int kPasses = (3 * BITS + 7) / 8;
+    __shared__ uint32_t h[kPasses][kRadix];
+    for (int j = threadIdx.x; j < kPasses * kRadix; j += kCountThreads) (&h[0][0])[j] = 0u;
+    __syncthreads();
+    for (size_t b = (size_t)blockIdx.x * kCountThreads; b < n; b += (size_t)gridDim.x * kCountThreads) {
+        const size_t i = b + threadIdx.x;
+        K k = 0;
+        if (i < n) keys[i] = k = mortonCode<K, BITS>(centroids[i], bounds);
+        countDigits<K>(k, i < n, kPasses, h);
+    }
+    __syncthreads();
+    flushDigits(kPasses, h, hist);
+}
+
+// A build's scratch before its first kernel: centroid bounds, digit counts, tickets and
+// first look-back array of the sort, and the fit's visit counters.
+struct BuildInit {
+    uint32_t* bounds;
+    uint4* sortHead;  // 16-byte words of the sort scratch to clear
+    size_t sortWords;
+    uint4* flags;
+    size_t flagWords;
+};
+__global__ void __launch_bounds__(256) buildInitKernel(BuildInit I) {
+    const size_t at = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    if (at < 6) I.bounds[at] = at < 3 ? 0xFFFFFFFFu : 0u;  // running minima start at the top, maxima at the bottom
+    for (size_t i = at; i < I.sortWords; i += step) I.sortHead[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (size_t i = at; i < I.flagWords; i += step) I.flags[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // One thread per internal node i in [0, n-2].
@@ -676,20 +807,23 @@ static grtError sortAndEmit(Context* ctx, BvhObject* o, const BuildLayout& L, ch
     const uint32_t n = o->leafCount;
     const float4* cen = (const float4*)(temp + L.centroids);
     const uint32_t* bounds = (const uint32_t*)(temp + L.bounds);
-    void* k0 = temp + L.keys[0];
-    uint32_t* v0 = (uint32_t*)(temp + L.vals[0]);
-    if (o->mortonBits == 30)
-        mortonKernel<uint32_t, 10><<<ceilDiv(n, 256), 256, 0, s>>>(cen, n, bounds, (uint32_t*)k0, v0);
-    else
-        mortonKernel<unsigned long long, 21><<<ceilDiv(n, 256), 256, 0, s>>>(cen, n, bounds, (unsigned long long*)k0,
-                                                                            v0);
-    GRT_LAUNCH_CHECK();
-    noteLaunches(1);
-    int fb = 0;
-    grtError err = radixSort(ctx, temp + L.keys[0], temp + L.keys[1], (uint32_t*)(temp + L.vals[0]),
-                             (uint32_t*)(temp + L.vals[1]), n, L.keyBytes, (int)o->mortonBits, (uint32_t*)(temp + L.hist),
-                             s, &fb);
+    const SortScratch S = sortScratch(temp + L.hist, n);
+    uint32_t* const vals[2] = {(uint32_t*)(temp + L.vals[0]), (uint32_t*)(temp + L.vals[1])};
+    grtError err;
+    if (o->mortonBits == 30) {
+        uint32_t* const keys[2] = {(uint32_t*)(temp + L.keys[0]), (uint32_t*)(temp + L.keys[1])};
+        mortonKernel<uint32_t, 10><<<countBlocks(ctx, n), kCountThreads, 0, s>>>(cen, n, bounds, keys[0], S.hist);
+        err = sortPasses<uint32_t>(ctx, keys, vals, n, L.passes, S, true, s);
+    } else {
+        unsigned long long* const keys[2] = {(unsigned long long*)(temp + L.keys[0]),
+                                             (unsigned long long*)(temp + L.keys[1])};
+        mortonKernel<unsigned long long, 21><<<countBlocks(ctx, n), kCountThreads, 0, s>>>(cen, n, bounds, keys[0],
+                                                                                         S.hist);
+        err = sortPasses<unsigned long long>(ctx, keys, vals, n, L.passes, S, true, s);
+    }
     if (err != GRT_SUCCESS) return err;
+    noteLaunches(1);
+    const int fb = L.finalBuf;
     const void* sk = temp + L.keys[fb];
     if (n >= 2 && emit) {
         if (o->mortonBits == 30)
@@ -706,10 +840,18 @@ static grtError sortAndEmit(Context* ctx, BvhObject* o, const BuildLayout& L, ch
     return GRT_SUCCESS;
 }
 
-static grtError resetBuildScratch(const BuildLayout& L, char* temp, uint32_t n, cudaStream_t s) {
-    GRT_CUDA(cudaMemsetAsync(temp + L.bounds, 0xFF, 12, s));       // running minima start at the top
-    GRT_CUDA(cudaMemsetAsync(temp + L.bounds + 12, 0x00, 12, s));  // running maxima start at the bottom
-    GRT_CUDA(cudaMemsetAsync(temp + L.flags, 0, 4 * (size_t)std::max(n, 1u), s));
+static grtError resetBuildScratch(Context* ctx, const BuildLayout& L, char* temp, uint32_t n, bool sorts,
+                                  cudaStream_t s) {
+    BuildInit I;
+    I.bounds = (uint32_t*)(temp + L.bounds);
+    I.sortHead = (uint4*)(temp + L.hist);
+    I.sortWords = sorts ? (kSortHeadBytes + lookBytes(n)) / sizeof(uint4) : 0;
+    I.flags = (uint4*)(temp + L.flags);
+    I.flagWords = alignUp(4 * (size_t)std::max(n, 1u), 16) / sizeof(uint4);
+    const size_t words = std::max(I.sortWords, I.flagWords);
+    buildInitKernel<<<std::min(ceilDiv(words, 256), 8u * (unsigned)std::max(1, smCount(ctx))), 256, 0, s>>>(I);
+    GRT_LAUNCH_CHECK();
+    noteLaunches(1);
     return GRT_SUCCESS;
 }
 
@@ -1004,7 +1146,7 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
                                    const BuildLayout& L, char* t, const PrimSource& S, cudaStream_t s,
                                    uint32_t radius = 0) {
     const uint32_t n = o->leafCount;
-    grtError e = resetBuildScratch(L, t, n, s);
+    grtError e = resetBuildScratch(c, L, t, n, op == GRT_BUILD_OPERATION_BUILD, s);
     if (e != GRT_SUCCESS) return e;
     const uint32_t* sorted = nullptr;
     if (op == GRT_BUILD_OPERATION_BUILD) {
@@ -1012,7 +1154,8 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
             e = launchSplit(c, o, L, t, S, radius, s);
             if (e != GRT_SUCCESS) return e;
         } else {
-            primCentroidKernel<<<ceilDiv(n, 256), 256, 0, s>>>(S, (float4*)(t + L.centroids),
+            const unsigned blocks = std::min(ceilDiv(n, 256), 8u * (unsigned)std::max(1, smCount(c)));
+            primCentroidKernel<<<blocks, 256, 0, s>>>(S, (float4*)(t + L.centroids),
                                                                (uint32_t*)(t + L.bounds));
             GRT_LAUNCH_CHECK();
             noteLaunches(1);
@@ -1342,7 +1485,7 @@ grtError grtBuildScene(grtContext ctx, uint32_t op, const grtSceneBuildInput* in
         o->built = true;
         return GRT_SUCCESS;
     }
-    e = resetBuildScratch(L, t, n, s);
+    e = resetBuildScratch(c, L, t, n, true, s);
     if (e != GRT_SUCCESS) return e;
     instanceSetupKernel<<<ceilDiv(n, 128), 128, 0, s>>>(I);
     GRT_LAUNCH_CHECK();
@@ -1396,10 +1539,10 @@ grtError grtSortPairs(grtContext ctx, void* keys, uint32_t* values, uint32_t cou
     char* t = (char*)temp;
     void* k1 = t;
     uint32_t* v1 = (uint32_t*)(t + alignUp(kb * count, 256));
-    uint32_t* hist = (uint32_t*)(t + alignUp(kb * count, 256) + alignUp(4 * (size_t)count, 256));
+    void* scratch = t + alignUp(kb * count, 256) + alignUp(4 * (size_t)count, 256);
     cudaStream_t s = (cudaStream_t)stream;
     int fb = 0;
-    grtError e = radixSort(asContext(ctx), keys, k1, values, v1, count, (int)kb, (int)significantBits, hist, s, &fb);
+    grtError e = radixSort(asContext(ctx), keys, k1, values, v1, count, (int)kb, (int)significantBits, scratch, s, &fb);
     if (e != GRT_SUCCESS) return e;
     if (fb == 1) {
         GRT_CUDA(cudaMemcpyAsync(keys, k1, kb * count, cudaMemcpyDeviceToDevice, s));

@@ -173,7 +173,7 @@ struct BuildLayout {
     size_t centroids;    // float4 per prim
     size_t keys[2];      // ping-pong keys
     size_t vals[2];      // ping-pong values
-    size_t hist;         // sort histogram / offsets
+    size_t hist;         // sort scratch: digit counts, tickets, look-back words
     size_t flags;        // fit visit counters
     size_t extra;        // scene: instance world boxes and records
     size_t total;
@@ -187,7 +187,7 @@ uint32_t resolveMortonBits(uint32_t count, const grtBuildOptions* opt);
 // Radix sort (build.cu).
 size_t sortScratchBytes(uint32_t count);
 grtError radixSort(Context* ctx, void* keys0, void* keys1, uint32_t* vals0, uint32_t* vals1, uint32_t count,
-                   int keyBytes, int significantBits, uint32_t* hist, cudaStream_t stream, int* finalBuf);
+                   int keyBytes, int significantBits, void* scratch, cudaStream_t stream, int* finalBuf);
 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ uint32_t floatToOrdered(float f) {
