@@ -15,6 +15,7 @@
 #include <unordered_map>
 
 #include "cluster.cuh"
+#include "emit_fit.cuh"
 #include "lbvh_block.cuh"
 #include "ploc.cuh"
 #include "split.cuh"
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kCountThreads) mortonKernel(const float4* __re
 }
 
 // A build's scratch before its first kernel: centroid bounds, digit counts, tickets and
-// first look-back array of the sort, and the fit's visit counters.
+// first look-back array of the sort, and the fit's visit counters (only of a fit that counts).
 struct BuildInit {
     uint32_t* bounds;
     uint4* sortHead;  // 16-byte words of the sort scratch to clear
@@ -418,15 +419,8 @@ __global__ void __launch_bounds__(256) buildInitKernel(BuildInit I) {
     for (size_t i = at; i < I.flagWords; i += step) I.flags[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// One thread per internal node i in [0, n-2].
-template <typename K>
-__global__ void __launch_bounds__(256) karrasKernel(const K* __restrict__ keys, int n, float4* __restrict__ nodes,
-                                                    uint32_t* __restrict__ parents) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n - 1) karrasNode<false>(keys, n, i, nodes, parents);
-}
-
-template <int KIND>  // 0 triangles, 1 AABB list, 2 instances
+// The fit of a hierarchy that is already there (refits, clustering builds, one primitive).
+template <int KIND>  // 0 triangles, 1 AABB list
 __global__ void __launch_bounds__(256) fitKernel(FitParams P) {
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < P.n) fitLeaf<KIND>(P, k);
@@ -439,10 +433,34 @@ __global__ void __launch_bounds__(256) quantizeKernel(const float4* wide, uint32
 }
 
 // The 8-wide node of each of the m binary nodes of an n-primitive tree (the
-// GRT_BUILD_WIDE8_NODES layout).
-__global__ void __launch_bounds__(256) wide8Kernel(const float4* nodes, uint32_t n, uint32_t m, float4* w8) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < m) wide8Node(nodes, n, k, w8);
+// GRT_BUILD_WIDE8_NODES layout). Slots 4s .. 4s+3 are those of child s's 4-wide node, or a
+// leaf child and three empty slots, so every row of an 8-wide node is a row of a 4-wide
+// one: one thread per row copies it, with whole lines read and written (12 us at 131,072
+// triangles; a thread per node that gathered up to seven binary nodes took 18).
+__global__ void __launch_bounds__(256) wide8Kernel(const float4* __restrict__ nodes, const float4* __restrict__ wide,
+                                                   uint32_t n, uint32_t m, float4* __restrict__ w8) {
+    const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t k = q / kWide8Words;
+    if (k >= m) return;
+    const uint32_t r = (uint32_t)(q % kWide8Words);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < 14) {
+        const bool words = r >= 12;
+        const uint32_t half = r & 1u, row = words ? 6u : 2 * (r >> 2) + ((r >> 1) & 1u);  // of the 4-wide node
+        const uint32_t c = reinterpret_cast<const uint32_t*>(nodes + 4 * k + 3)[half];
+        const float none = words ? __uint_as_float(kInvalid) : (row & 1u) ? -INFINITY : INFINITY;
+        if (n == 1 && half == 1) {
+            o = make_float4(none, none, none, none);
+        } else if (c & kLeafBit) {  // binary rows: (lo, hi) of child 0, then of child 1
+            const float own =
+                words ? __uint_as_float(c)
+                      : reinterpret_cast<const float*>(nodes + 4 * k + (row >> 1))[2 * half + (row & 1u)];
+            o = make_float4(own, none, none, none);
+        } else {
+            o = wide[kWideWords * (size_t)c + row];
+        }
+    }
+    w8[q] = o;
 }
 
 // The extra node formats of object o, after its fit.
@@ -454,8 +472,8 @@ static grtError launchNodeFormats(const BvhObject* o, cudaStream_t s) {
         noteLaunches(1);
     }
     if (o->w8nodes) {
-        wide8Kernel<<<ceilDiv(o->nodeCount, 256), 256, 0, s>>>((const float4*)o->nodes, o->leafCount, o->nodeCount,
-                                                               (float4*)o->w8nodes);
+        wide8Kernel<<<ceilDiv((size_t)o->nodeCount * kWide8Words, 256), 256, 0, s>>>(
+            (const float4*)o->nodes, (const float4*)o->wide, o->leafCount, o->nodeCount, (float4*)o->w8nodes);
         GRT_LAUNCH_CHECK();
         noteLaunches(1);
     }
@@ -801,9 +819,8 @@ static void destroyBvhObject(BvhObject* o) {
     delete o;
 }
 
-// Morton + sort + Karras over the centroids already in temp (count >= 1).
-static grtError sortAndEmit(Context* ctx, BvhObject* o, const BuildLayout& L, char* temp, cudaStream_t s,
-                            const uint32_t** sortedOut, bool emit = true, const void** sortedKeysOut = nullptr) {
+// Morton codes and their sort over the centroids already in temp (count >= 1).
+static grtError sortCodes(Context* ctx, BvhObject* o, const BuildLayout& L, char* temp, cudaStream_t s) {
     const uint32_t n = o->leafCount;
     const float4* cen = (const float4*)(temp + L.centroids);
     const uint32_t* bounds = (const uint32_t*)(temp + L.bounds);
@@ -823,32 +840,64 @@ static grtError sortAndEmit(Context* ctx, BvhObject* o, const BuildLayout& L, ch
     }
     if (err != GRT_SUCCESS) return err;
     noteLaunches(1);
-    const int fb = L.finalBuf;
-    const void* sk = temp + L.keys[fb];
-    if (n >= 2 && emit) {
-        if (o->mortonBits == 30)
-            karrasKernel<uint32_t><<<ceilDiv(n - 1, 256), 256, 0, s>>>((const uint32_t*)sk, (int)n,
-                                                                        (float4*)o->nodes, (uint32_t*)o->parents);
-        else
-            karrasKernel<unsigned long long><<<ceilDiv(n - 1, 256), 256, 0, s>>>(
-                (const unsigned long long*)sk, (int)n, (float4*)o->nodes, (uint32_t*)o->parents);
-        GRT_LAUNCH_CHECK();
-        noteLaunches(1);
-    }
-    *sortedOut = (const uint32_t*)(temp + L.vals[fb]);
-    if (sortedKeysOut) *sortedKeysOut = sk;
     return GRT_SUCCESS;
 }
 
+// The emission's lists: those of the first launch's blocks, then of each further launch's.
+static uint32_t emitLists(uint32_t n) {
+    uint32_t total = 0;
+    for (uint32_t lists = ceilDiv(std::max(n, 1u), kEmitLeaves);; lists = ceilDiv(lists, kTopFan)) {
+        total += lists;
+        if (lists == 1) return total;
+    }
+}
+size_t emitTopBytes(uint32_t n) { return (size_t)emitLists(n) * (kTopMax * sizeof(uint4) + sizeof(uint4)); }
+
+// Emission and fit over the sorted codes (P.n >= 2, P.sortedPrims their order).
+template <typename K, int KIND>
+static grtError launchEmitFitT(Context* c, BvhObject* o, const BuildLayout& L, char* temp, const FitParams& P,
+                               cudaStream_t s) {
+    EmitParams E;
+    E.fit = P;
+    E.parents = (uint32_t*)o->parents;
+    const K* keys = (const K*)(temp + L.keys[L.finalBuf]);
+    grtError e = allowSmem(emitTopKernel<K, KIND>, sizeof(TopShared));
+    if (e != GRT_SUCCESS) return e;
+    uint32_t lists = ceilDiv(P.n, kEmitLeaves);
+    TopLists in;
+    in.tops = (uint4*)(temp + L.tops);
+    in.counts = (uint32_t*)(in.tops + (size_t)emitLists(P.n) * kTopMax);
+    emitFitKernel<K, KIND><<<lists, kEmitLeaves, 0, s>>>(E, keys, in);
+    noteLaunches(1);
+    while (lists > 1) {
+        const TopLists out{in.tops + (size_t)lists * kTopMax, in.counts + lists};
+        const uint32_t next = ceilDiv(lists, kTopFan);
+        emitTopKernel<K, KIND><<<next, kTopThreads, sizeof(TopShared), s>>>(E, keys, in, lists, out,
+                                                                           &workspace(c)->error);
+        noteLaunches(1);
+        in = out;
+        lists = next;
+    }
+    GRT_LAUNCH_CHECK();
+    return GRT_SUCCESS;
+}
+
+template <int KIND>
+static grtError launchEmitFit(Context* c, BvhObject* o, const BuildLayout& L, char* temp, const FitParams& P,
+                              cudaStream_t s) {
+    return o->mortonBits == 30 ? launchEmitFitT<uint32_t, KIND>(c, o, L, temp, P, s)
+                               : launchEmitFitT<unsigned long long, KIND>(c, o, L, temp, P, s);
+}
+
 static grtError resetBuildScratch(Context* ctx, const BuildLayout& L, char* temp, uint32_t n, bool sorts,
-                                  cudaStream_t s) {
+                                  bool counts, cudaStream_t s) {
     BuildInit I;
     I.bounds = (uint32_t*)(temp + L.bounds);
     I.sortHead = (uint4*)(temp + L.hist);
     I.sortWords = sorts ? (kSortHeadBytes + lookBytes(n)) / sizeof(uint4) : 0;
     I.flags = (uint4*)(temp + L.flags);
-    I.flagWords = alignUp(4 * (size_t)std::max(n, 1u), 16) / sizeof(uint4);
-    const size_t words = std::max(I.sortWords, I.flagWords);
+    I.flagWords = counts ? alignUp(4 * (size_t)std::max(n, 1u), 16) / sizeof(uint4) : 0;
+    const size_t words = std::max<size_t>(std::max(I.sortWords, I.flagWords), 6);
     buildInitKernel<<<std::min(ceilDiv(words, 256), 8u * (unsigned)std::max(1, smCount(ctx))), 256, 0, s>>>(I);
     GRT_LAUNCH_CHECK();
     noteLaunches(1);
@@ -1146,7 +1195,8 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
                                    const BuildLayout& L, char* t, const PrimSource& S, cudaStream_t s,
                                    uint32_t radius = 0) {
     const uint32_t n = o->leafCount;
-    grtError e = resetBuildScratch(c, L, t, n, op == GRT_BUILD_OPERATION_BUILD, s);
+    const bool emits = op == GRT_BUILD_OPERATION_BUILD && radius == 0 && n >= 2;
+    grtError e = resetBuildScratch(c, L, t, n, op == GRT_BUILD_OPERATION_BUILD, !emits, s);
     if (e != GRT_SUCCESS) return e;
     const uint32_t* sorted = nullptr;
     if (op == GRT_BUILD_OPERATION_BUILD) {
@@ -1160,9 +1210,10 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
             GRT_LAUNCH_CHECK();
             noteLaunches(1);
         }
-        const void* sortedKeys = nullptr;
-        e = sortAndEmit(c, o, L, t, s, &sorted, radius == 0, &sortedKeys);
+        e = sortCodes(c, o, L, t, s);
         if (e != GRT_SUCCESS) return e;
+        sorted = (const uint32_t*)(t + L.vals[L.finalBuf]);
+        const void* sortedKeys = t + L.keys[L.finalBuf];
         if (radius == kSubtreeMethod && n >= 2) {
             e = launchSubtreeCluster(c, o, L, t, S, sorted, sortedKeys, s);
             if (e != GRT_SUCCESS) return e;
@@ -1182,6 +1233,12 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
     P.parents = (const uint32_t*)o->parents;
     P.flags = (uint32_t*)(t + L.flags);
     P.header = o->dHeader;
+    if (emits) {
+        e = input->type == GRT_PRIMITIVE_TRIANGLE_MESH ? launchEmitFit<0>(c, o, L, t, P, s)
+                                                       : launchEmitFit<1>(c, o, L, t, P, s);
+        if (e != GRT_SUCCESS) return e;
+        return launchNodeFormats(o, s);
+    }
     if (input->type == GRT_PRIMITIVE_TRIANGLE_MESH)
         fitKernel<0><<<ceilDiv(n, 256), 256, 0, s>>>(P);
     else
@@ -1485,29 +1542,25 @@ grtError grtBuildScene(grtContext ctx, uint32_t op, const grtSceneBuildInput* in
         o->built = true;
         return GRT_SUCCESS;
     }
-    e = resetBuildScratch(c, L, t, n, true, s);
+    e = resetBuildScratch(c, L, t, n, true, false, s);
     if (e != GRT_SUCCESS) return e;
     instanceSetupKernel<<<ceilDiv(n, 128), 128, 0, s>>>(I);
     GRT_LAUNCH_CHECK();
     noteLaunches(1);
-    const uint32_t* sorted = nullptr;
-    e = sortAndEmit(c, o, L, t, s, &sorted);
+    e = sortCodes(c, o, L, t, s);
     if (e != GRT_SUCCESS) return e;
     FitParams P{};
     P.n = n;
-    P.sortedPrims = sorted;
+    P.sortedPrims = (const uint32_t*)(t + L.vals[L.finalBuf]);
     P.nodes = (float4*)o->nodes;
     P.wide = (float4*)o->wide;
     P.leaves = o->leaves;
-    P.parents = (const uint32_t*)o->parents;
-    P.flags = (uint32_t*)(t + L.flags);
     P.header = o->dHeader;
     P.primToLeaf = o->primToLeaf;
     P.instBoxes = I.boxes;
     P.instRecords = I.records;
-    fitKernel<2><<<ceilDiv(n, 256), 256, 0, s>>>(P);
-    GRT_LAUNCH_CHECK();
-    noteLaunches(1);
+    e = launchEmitFit<2>(c, o, L, t, P, s);
+    if (e != GRT_SUCCESS) return e;
     e = launchNodeFormats(o, s);
     if (e != GRT_SUCCESS) return e;
     o->built = true;

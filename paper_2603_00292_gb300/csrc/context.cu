@@ -131,6 +131,7 @@ BuildLayout buildLayout(uint32_t count, uint32_t mortonBits, bool scene) {
     L.vals[1] = take(4 * n);
     L.hist = take(sortScratchBytes(count));
     L.flags = take(4 * n);
+    L.tops = take(emitTopBytes(count));
     L.extra = scene ? take(32 * n + sizeof(InstanceRecord) * n) : off;
     L.total = off;
     return L;

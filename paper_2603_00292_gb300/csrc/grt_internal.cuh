@@ -175,6 +175,7 @@ struct BuildLayout {
     size_t vals[2];      // ping-pong values
     size_t hist;         // sort scratch: digit counts, tickets, look-back words
     size_t flags;        // fit visit counters
+    size_t tops;         // lists of subtrees between the launches of the emission (emit_fit.cuh)
     size_t extra;        // scene: instance world boxes and records
     size_t total;
     int passes;          // radix passes
@@ -183,6 +184,9 @@ struct BuildLayout {
 };
 BuildLayout buildLayout(uint32_t count, uint32_t mortonBits, bool scene);
 uint32_t resolveMortonBits(uint32_t count, const grtBuildOptions* opt);
+
+// Bytes of the emission's lists for n leaves (build.cu).
+size_t emitTopBytes(uint32_t n);
 
 // Radix sort (build.cu).
 size_t sortScratchBytes(uint32_t count);

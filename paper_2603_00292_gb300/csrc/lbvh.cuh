@@ -265,6 +265,20 @@ __device__ __forceinline__ void writeChildBox(float4* nodes, uint32_t p, uint32_
     n2[2 * 2 + side] = make_float2(b.lo.z, b.hi.z);
 }
 
+// Leaf record k of triangle (or reference) `item` with vertices v, and its ID's leaf position.
+__device__ __forceinline__ void writeTriangleLeaf(const FitParams& P, uint32_t k, uint32_t item, const float3 v[3]) {
+    bool owner = true;
+    const uint32_t prim = P.src.kind == 2 ? refTriangle(P.src, item, &owner) : item;
+    float4* rec = reinterpret_cast<float4*>(P.leaves) + 3 * (size_t)k;
+    rec[0] = make_float4(v[0].x, v[0].y, v[0].z, __uint_as_float(prim));
+    // w slots: L1 norms of the edges v1-v0 and v2-v0 (scale of the traversal's error bounds)
+    const float e1 = fabsf(v[1].x - v[0].x) + fabsf(v[1].y - v[0].y) + fabsf(v[1].z - v[0].z);
+    const float e2 = fabsf(v[2].x - v[0].x) + fabsf(v[2].y - v[0].y) + fabsf(v[2].z - v[0].z);
+    rec[1] = make_float4(v[1].x, v[1].y, v[1].z, e1);
+    rec[2] = make_float4(v[2].x, v[2].y, v[2].z, e2);
+    if (owner) P.primToLeaf[prim] = k;
+}
+
 // Slots 2t and 2t+1 of 4-wide node w: two boxes (a, b) and their child words (kNone
 // with an empty box for an empty slot). Layout of a wide node (kWideWords float4): lo.x
 // of slots 0-3, hi.x, lo.y, hi.y, lo.z, hi.z, the four child words, then one unused
@@ -462,19 +476,11 @@ template <int KIND, bool BLOCK = false>  // KIND: 0 triangles, 1 AABB list, 2 in
 __device__ __forceinline__ void fitLeaf(const FitParams& P, uint32_t k, uint32_t* blockFlags = nullptr) {
     Box3 b;
     if (KIND == 0) {
-        float4* rec = reinterpret_cast<float4*>(P.leaves) + 3 * (size_t)k;
+        const float4* rec = reinterpret_cast<const float4*>(P.leaves) + 3 * (size_t)k;
         const uint32_t item = P.sortedPrims ? __ldcg(P.sortedPrims + k) : __float_as_uint(rec[0].w);
         float3 v[3];
         b = primBox(P.src, item, v);
-        bool owner = true;
-        const uint32_t prim = P.src.kind == 2 ? refTriangle(P.src, item, &owner) : item;
-        rec[0] = make_float4(v[0].x, v[0].y, v[0].z, __uint_as_float(prim));
-        // w slots: L1 norms of the edges v1-v0 and v2-v0 (scale of the traversal's error bounds)
-        const float e1 = fabsf(v[1].x - v[0].x) + fabsf(v[1].y - v[0].y) + fabsf(v[1].z - v[0].z);
-        const float e2 = fabsf(v[2].x - v[0].x) + fabsf(v[2].y - v[0].y) + fabsf(v[2].z - v[0].z);
-        rec[1] = make_float4(v[1].x, v[1].y, v[1].z, e1);
-        rec[2] = make_float4(v[2].x, v[2].y, v[2].z, e2);
-        if (owner) P.primToLeaf[prim] = k;
+        writeTriangleLeaf(P, k, item, v);
     } else if (KIND == 1) {
         uint32_t* ids = reinterpret_cast<uint32_t*>(P.leaves);
         const uint32_t prim = P.sortedPrims ? __ldcg(P.sortedPrims + k) : ids[k];
