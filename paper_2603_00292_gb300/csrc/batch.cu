@@ -175,10 +175,12 @@ struct ChunkRaySource {
     const TraceParams* P;
     uint32_t base, n;
     __device__ unsigned long long count() const { return n; }
+    __device__ uint32_t warps() const { return blockDim.x >> 5; }  // one block takes the chunk
     __device__ bool begin(uint32_t i, const TraceParams& Q, Stack& st, RayState& s) const {
         const size_t r = (size_t)base + i;
         const float4 a = Q.rays[2 * r], b = Q.rays[2 * r + 1];
-        beginRay<false>(Q, st, s, f3(a), f3(b), a.w, b.w);
+        beginRay<false, true>(Q, st, s, f3(a), f3(b), a.w, b.w);
+        if (s.next != kNone && !meetsRoot<true>(Q, s)) s.next = kNone;
         return true;
     }
     __device__ void finish(uint32_t i, const RayState& s) const { storeHit(P->hits, base + i, s.best); }
@@ -193,6 +195,7 @@ __device__ __noinline__ void traceChunk(const BatchParams& B, const BatchSceneDe
     P.target.primType = GRT_PRIMITIVE_TRIANGLE_MESH;
     P.target.geomType = 0;
     P.target.empty = S.n == 0;
+    P.root = S.header;
     P.rays = S.rayBuf;
     P.hits = S.hitBuf;
     P.count = S.rays;
@@ -544,10 +547,17 @@ grtError grtCreateBatch(grtContext ctx, const grtBatchScene* scenes, uint32_t sc
     b->sceneCount = sceneCount;
     b->itemCount = (uint32_t)items.size();
     b->blockSize = bs;
-    const size_t stackSmem = (size_t)bs * traceSmemWords(opt.sharedStackDepth) * 4;
+    const size_t stackSmem = (size_t)bs * traceSmemWords(false, false, opt.sharedStackDepth) * 4;
     const size_t sortSmem = ((size_t)warps * kBlockRadix + 2 * kBlockRadix) * 4;
     const size_t clusterSmem = (size_t)warps * sizeof(ClusterWarpList);
     b->smem = std::max<size_t>(std::max(std::max(stackSmem, sortSmem), clusterSmem), 33 * 4);
+    if (b->smem > 48 * 1024 &&
+        cudaFuncSetAttribute(batchKernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)std::max<size_t>(b->smem, 256 * traceSmemWords(false, false, 32) * 4)) != cudaSuccess) {
+        cudaGetLastError();
+        delete b;
+        return GRT_ERROR_CUDA;
+    }
     int perSm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, batchKernel, (int)bs, b->smem) != cudaSuccess ||
         perSm < 1)

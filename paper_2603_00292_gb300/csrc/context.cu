@@ -26,7 +26,7 @@ struct Context {
 unsigned long long* nextCounter(Context* c) {
     std::lock_guard<std::mutex> g(c->lock);
     const unsigned slot = c->nextSlot++ % kCounterSlots;
-    return &c->dWork->counters[slot];
+    return c->dWork->counters[slot];
 }
 
 grtError contextAux(Context* c, size_t bytes, void** ptr) {

@@ -73,7 +73,8 @@ struct DeviceWorkspace {
     uint32_t error;
     uint32_t pad[31];
     unsigned long long stats[16];  // traversal statistics (grtTraceStatistics order)
-    unsigned long long counters[kCounterSlots];  // per-launch work counters (round robin)
+    // per-launch work counters (round robin): items taken, blocks done; zero between launches
+    unsigned long long counters[kCounterSlots][2];
 };
 
 // ------------------------------------------------------------------ host helpers
@@ -108,7 +109,7 @@ inline unsigned ceilDiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b)
 struct Context;
 Context* asContext(grtContext c);
 DeviceWorkspace* workspace(Context* c);
-unsigned long long* nextCounter(Context* c);  // a zeroed-on-use work counter slot
+unsigned long long* nextCounter(Context* c);  // a work counter slot, zero (kernels leave theirs at zero)
 // Caller-or-context global stack memory for traversal spills (grown on demand).
 grtError contextScratch(Context* c, size_t bytes, void** ptr);
 // Context memory for buffers one call passes between its own launches (grown on demand;

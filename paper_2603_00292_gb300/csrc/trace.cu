@@ -13,13 +13,28 @@ namespace grt {
 
 // FM: the node formats the walk may meet (traverse.cuh): kFmPlain (4-wide only),
 // kFmQuant (4-wide or quantised, read per level) or kFmWide8 (8-wide on every level).
-template <bool ANY, bool SCENE, bool COUNT, int FM = kFmPlain>
-__global__ void traceKernel(TraceParams P) {
+//
+// PHASED: of a closest hit, the phased form of refillLoop; without it the per-ray form, for
+// 4-slot nodes of one geometry (kPerRayFrom).
+//
+// Register caps, measured on 4 M rays through 1 M spheres and 64 terrains (us). One geometry,
+// closest per ray: 72 (3,860; 64: 4,160, 76: 4,195, 80: 4,160, 96: 4,580, none: 5,290); any hit:
+// 64 (2,345; 56: 2,570, 68: 2,470, 96: 2,750). Both spill a few words outside the loop's
+// common path for 7 and 8 blocks of 128 threads on an SM instead of 4 and 5. Scenes hold
+// twice the state (the world ray and the level's) and 8-slot visits twice the distances:
+// closest 128 (64 terrains near 592; 104: 655, 96: 648).
+__host__ __device__ constexpr int traceRegisters(bool any, bool scene, int w, bool phased) {
+    return scene ? 128 : any ? (w == 8 ? 96 : 64) : phased ? 128 : 72;
+}
+
+template <bool ANY, bool SCENE, bool COUNT, int FM = kFmPlain, bool PHASED = true>
+__global__ void __maxnreg__(traceRegisters(ANY, SCENE, slotsOf(FM), PHASED)) traceKernel(TraceParams P) {
     extern __shared__ uint32_t sstack[];
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     Stack st{sstack + threadIdx.x, P.globalStack + gtid, P.sharedDepth, P.globalDepth, P.globalStride, 0};
-    RayBufferSource<SCENE> src{P.count, &P};
-    refillLoop<ANY, SCENE, COUNT, FM>(P, st, src);
+    RayBufferSource<ANY, SCENE> src{P.count, &P};
+    refillLoop<ANY, SCENE, COUNT, FM, PHASED>(P, st, src);
+    releaseCounter(P.counter);
 }
 
 // The closest hits' t, u, v recomputed in double-float, one thread per ray after traversal so
@@ -113,7 +128,9 @@ __global__ void aoCompactKernel(TraceParams P, uint32_t pixels, uint32_t* __rest
 }
 
 // Items = (listed pixel, sample); the ray comes from the pixel's stored frame.
-struct AoSource {
+struct AoSource : GridSource {
+    __device__ AoSource(const TraceParams* P_, const uint32_t* l, const uint32_t* c, uint32_t* o, const float4* f)
+        : P(P_), list(l), listCount(c), counts(o), frames(f) {}
     const TraceParams* P;
     const uint32_t* list;
     const uint32_t* listCount;
@@ -127,7 +144,7 @@ struct AoSource {
         AoFrame F;
         F.org = f3(a), F.n = f3(b), F.tg = f3(c);
         F.bt = cross3(F.n, F.tg);
-        beginRay<true>(Pm, st, s, F.org, aoDirection(F, Pm.seed, list[slot], smp), 0.0f, Pm.aoLength);
+        beginRay<true, true>(Pm, st, s, F.org, aoDirection(F, Pm.seed, list[slot], smp), 0.0f, Pm.aoLength);
         return true;
     }
     __device__ void finish(uint32_t i, const RayState& s) const {
@@ -148,6 +165,7 @@ __global__ void __maxnreg__(GRT_AO_MAXNREG) aoTraceKernel(TraceParams P, const u
     Stack st{sstack + threadIdx.x, P.globalStack + gtid, P.sharedDepth, P.globalDepth, P.globalStride, 0};
     AoSource src{&P, list, listCount, counts, frames};
     refillLoop<true, true, COUNT, FM>(P, st, src);
+    releaseCounter(P.counter);
 }
 
 __global__ void aoFinishKernel(const uint32_t* __restrict__ list, const uint32_t* __restrict__ listCount,
@@ -244,7 +262,8 @@ __device__ __forceinline__ float3 shadeColour(const ShadeParams& S, const ShadeH
 
 // Items = pixels; a lit hit pixel traces its shadow ray, everything else is written at once.
 template <bool SCENE>
-struct ShadowSource {
+struct ShadowSource : GridSource {
+    __device__ explicit ShadowSource(const ShadeParams* S_) : S(S_) {}
     const ShadeParams* S;
     __device__ unsigned long long count() const { return S->n; }
     __device__ ShadeHit setup(uint32_t i) const {
@@ -258,7 +277,7 @@ struct ShadowSource {
             const ShadeHit H = setup(i);
             if (H.nl > 0.0f) {
                 const float3 l = make_float3(S->light[0], S->light[1], S->light[2]);
-                beginRay<SCENE>(P, st, s, (H.o + H.d * H.t) + H.nf * 1e-4f, l, 0.0f, INFINITY);
+                beginRay<SCENE, true>(P, st, s, (H.o + H.d * H.t) + H.nf * 1e-4f, l, 0.0f, INFINITY);
                 return true;
             }
         }
@@ -278,13 +297,15 @@ struct ShadowSource {
     }
 };
 
+// One geometry at 72 registers: a 1080p step 426 us, 439 at 80, 440 at 96, 454 at 64.
 template <bool SCENE, int FM = kFmPlain>
-__global__ void shadeForwardKernel(TraceParams P, ShadeParams S) {
+__global__ void __maxnreg__(SCENE ? 128 : 72) shadeForwardKernel(TraceParams P, ShadeParams S) {
     extern __shared__ uint32_t sstack[];
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     Stack st{sstack + threadIdx.x, P.globalStack + gtid, P.sharedDepth, P.globalDepth, P.globalStride, 0};
     ShadowSource<SCENE> src{&S};
     refillLoop<true, SCENE, false, FM>(P, st, src);
+    releaseCounter(P.counter);
 }
 
 // One pixel's share of the adjoint: dL/dc_k and dL/dv_k for the hit triangle's three
@@ -436,6 +457,7 @@ __global__ void shadeBackwardKernel(TraceParams P, ShadeParams S, uint32_t nv) {
             scatterAdjoint<PRIV>(A, priv, S, nv);
         }
     }
+    releaseCounter(P.counter);
     // light gradient: warp sum, one atomic per warp and axis
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -512,6 +534,11 @@ static LaunchShape persistentShape(Context* c, K kernel, int blockSize, size_t s
         if (it != cache.end()) perSm = it->second;
     }
     if (perSm == 0) {
+        // above 48 KB (deep stacks in large blocks) a kernel has to opt in: to the most any
+        // call can ask for, so that no later call lowers it
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)std::max<size_t>(smem, 256 * traceSmemWords(false, false, 32, 8) * sizeof(uint32_t)));
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, kernel, blockSize, smem) != cudaSuccess || perSm < 1)
             perSm = 1;
         std::lock_guard<std::mutex> g(m);
@@ -550,6 +577,7 @@ static grtError prepareTrace(Context* c, grtScene scene, grtGeometry geom, grtFu
     P.target.primType = o->primType;
     P.target.geomType = o->geomType;
     P.target.empty = o->primCount == 0;
+    P.root = o->dHeader;
     P.maxSteps = 1u << 26;  // far above any legitimate walk; stops a corrupted (cyclic) hierarchy
     P.rayMask = (opt && opt->rayMask) ? opt->rayMask : 0xFFFFFFFFu;
     const float compact = (opt && opt->compactThreshold > 0.f) ? fminf(opt->compactThreshold, 1.f) : defaultCompact;
@@ -605,6 +633,17 @@ static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int thre
     return e;
 }
 
+// Blocks of a trace of n items: a warp takes one at least (itemLanes). A caller's own stack
+// buffer that holds a block per blockSize items, but not these, keeps the grid to what it
+// holds.
+static int traceBlocks(const grtTraceOptions* opt, const TraceParams& P, LaunchShape L, uint32_t n) {
+    const int spread = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize / 32));
+    if (!opt || !opt->globalStack || P.globalDepth == 0) return spread;
+    const size_t fits = (opt->globalStackBytes & ~(size_t)255) / ((size_t)L.blockSize * P.globalDepth * sizeof(uint32_t));
+    const int least = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize));
+    return std::max(least, (int)std::min<size_t>(fits, (size_t)spread));
+}
+
 // The node formats a walk over P's target can meet (the kernel variant to launch): a
 // geometry's own format; an 8-wide scene walks 8-wide levels only (its instances must be
 // 8-wide); a 4-wide scene walks the 4-wide or quantised nodes of its instances, and can
@@ -616,14 +655,26 @@ static int walkFormats(const TraceParams& P, bool scene) {
     return kFmPlain;
 }
 
+// Rays from which closest hits in one geometry (4-slot nodes) take the per-ray form with its
+// 28 warps an SM instead of the phased one with 16. It has more work in flight; the phased
+// form has the shorter chain per ray, which is what a smaller launch waits for (us, per ray
+// against phased): 2 M camera rays 150 / 186, 1.9 M 388 / 437, 3 M through 1 M spheres 4,510 /
+// 4,570; 733,391 through 41,718 spheres 1,203 / 1,158, 303,000 68 / 61, 86,000 54 / 48.
+constexpr uint32_t kPerRayFrom = 1u << 20;
+
 template <bool ANY, bool COUNT>
-static void traceKernelFor(bool scene, int fm, void (**k)(TraceParams)) {
+static void traceKernelFor(bool scene, int fm, uint32_t n, void (**k)(TraceParams)) {
+    const bool perRay = !ANY && n >= kPerRayFrom;
     if (fm == kFmWide8)
         *k = scene ? traceKernel<ANY, true, COUNT, kFmWide8> : traceKernel<ANY, false, COUNT, kFmWide8>;
     else if (fm == kFmQuant)
-        *k = scene ? traceKernel<ANY, true, COUNT, kFmQuant> : traceKernel<ANY, false, COUNT, kFmQuant>;
+        *k = scene    ? traceKernel<ANY, true, COUNT, kFmQuant>
+             : perRay ? traceKernel<ANY, false, COUNT, kFmQuant, ANY>
+                      : traceKernel<ANY, false, COUNT, kFmQuant>;
     else
-        *k = scene ? traceKernel<ANY, true, COUNT> : traceKernel<ANY, false, COUNT>;
+        *k = scene    ? traceKernel<ANY, true, COUNT>
+             : perRay ? traceKernel<ANY, false, COUNT, kFmPlain, ANY>
+                      : traceKernel<ANY, false, COUNT>;
 }
 
 template <bool ANY>
@@ -643,17 +694,16 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
     P.count = n;
     void (*kernel)(TraceParams) = nullptr;
     if (count)
-        traceKernelFor<ANY, true>(isScene, walkFormats(P, isScene), &kernel);
+        traceKernelFor<ANY, true>(isScene, walkFormats(P, isScene), n, &kernel);
     else
-        traceKernelFor<ANY, false>(isScene, walkFormats(P, isScene), &kernel);
+        traceKernelFor<ANY, false>(isScene, walkFormats(P, isScene), n, &kernel);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t smem = (size_t)bs * traceSmemWords(P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
+    const size_t smem = (size_t)bs * traceSmemWords(ANY, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
-    L.blocks = std::min<int>(L.blocks, (int)ceilDiv(n, bs));
+    L.blocks = traceBlocks(opt, P, L, n);
     e = bindGlobalStack(c, opt, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);
-    GRT_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(unsigned long long), s));
     kernel<<<L.blocks, bs, smem, s>>>(P);
     if (!ANY) refineKernel<<<refineBlocks(n), 256, 0, s>>>(P);
     GRT_LAUNCH_CHECK();
@@ -732,18 +782,17 @@ grtError grtTraceClosestNoAlloc(grtContext ctx, grtScene scene, grtGeometry geom
     P.count = rayCount;
     void (*kernel)(TraceParams) = nullptr;
     if (count)
-        traceKernelFor<false, true>(isScene, walkFormats(P, isScene), &kernel);
+        traceKernelFor<false, true>(isScene, walkFormats(P, isScene), rayCount, &kernel);
     else
-        traceKernelFor<false, false>(isScene, walkFormats(P, isScene), &kernel);
-    const size_t smem = (size_t)bs * traceSmemWords(P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
+        traceKernelFor<false, false>(isScene, walkFormats(P, isScene), rayCount, &kernel);
+    const size_t smem = (size_t)bs * traceSmemWords(false, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
-    L.blocks = std::min<int>(L.blocks, (int)ceilDiv(rayCount, bs));
+    L.blocks = std::min<int>(L.blocks, (int)ceilDiv(rayCount, bs / 32));
     L.blocks = std::max(1, std::min<int>(L.blocks, (int)(capacity / perBlock)));  // the grid shrinks to fit
     P.counter = reinterpret_cast<unsigned long long*>(base);
     P.globalStack = reinterpret_cast<uint32_t*>(static_cast<char*>(base) + kNoAllocStackOffset);
     P.globalStride = (uint32_t)(L.blocks * bs);
     cudaStream_t s = (cudaStream_t)stream;
-    GRT_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(unsigned long long), s));  // the work counter starts at zero
     kernel<<<L.blocks, bs, smem, s>>>(P);
     refineKernel<<<refineBlocks(rayCount), 256, 0, s>>>(P);
     GRT_LAUNCH_CHECK();
@@ -760,25 +809,29 @@ grtError grtGetTraceGlobalStackSize(grtContext ctx, const grtTraceOptions* optio
     Context* c = asContext(ctx);
     int threads = 0;
     // every variant a launch may choose, each with its own shared memory
-    auto most = [&](auto k, int w) {
-        const size_t sm = (size_t)bs * traceSmemWords(sh, w) * sizeof(uint32_t);
+    auto most = [&](auto k, bool any, bool scene, int w) {
+        const size_t sm = (size_t)bs * traceSmemWords(any, scene, sh, w) * sizeof(uint32_t);
         threads = std::max(threads, persistentShape(c, k, bs, sm).blocks * bs);
     };
-    most(traceKernel<false, false, false>, 4), most(traceKernel<false, true, false>, 4);
-    most(traceKernel<true, false, false>, 4), most(traceKernel<true, true, false>, 4);
-    most(traceKernel<false, false, true>, 4), most(traceKernel<false, true, true>, 4);
-    most(traceKernel<true, false, true>, 4), most(traceKernel<true, true, true>, 4);
-    most(traceKernel<false, false, false, kFmWide8>, 8), most(traceKernel<false, true, false, kFmWide8>, 8);
-    most(traceKernel<true, false, false, kFmWide8>, 8), most(traceKernel<true, true, false, kFmWide8>, 8);
-    most(traceKernel<false, false, true, kFmWide8>, 8), most(traceKernel<false, true, true, kFmWide8>, 8);
-    most(traceKernel<true, false, true, kFmWide8>, 8), most(traceKernel<true, true, true, kFmWide8>, 8);
-    most(traceKernel<false, false, false, kFmQuant>, 4), most(traceKernel<false, true, false, kFmQuant>, 4);
-    most(traceKernel<true, false, false, kFmQuant>, 4), most(traceKernel<true, true, false, kFmQuant>, 4);
-    most(traceKernel<false, false, true, kFmQuant>, 4), most(traceKernel<false, true, true, kFmQuant>, 4);
-    most(traceKernel<true, false, true, kFmQuant>, 4), most(traceKernel<true, true, true, kFmQuant>, 4);
-    most(aoTraceKernel<false>, 4), most(aoTraceKernel<true>, 4);
-    most(aoTraceKernel<false, kFmWide8>, 8), most(aoTraceKernel<true, kFmWide8>, 8);
-    most(aoTraceKernel<false, kFmQuant>, 4), most(aoTraceKernel<true, kFmQuant>, 4);
+    most(traceKernel<false, false, false>, false, false, 4), most(traceKernel<false, true, false>, false, true, 4);
+    most(traceKernel<true, false, false>, true, false, 4), most(traceKernel<true, true, false>, true, true, 4);
+    most(traceKernel<false, false, true>, false, false, 4), most(traceKernel<false, true, true>, false, true, 4);
+    most(traceKernel<true, false, true>, true, false, 4), most(traceKernel<true, true, true>, true, true, 4);
+    most(traceKernel<false, false, false, kFmWide8>, false, false, 8), most(traceKernel<false, true, false, kFmWide8>, false, true, 8);
+    most(traceKernel<true, false, false, kFmWide8>, true, false, 8), most(traceKernel<true, true, false, kFmWide8>, true, true, 8);
+    most(traceKernel<false, false, true, kFmWide8>, false, false, 8), most(traceKernel<false, true, true, kFmWide8>, false, true, 8);
+    most(traceKernel<true, false, true, kFmWide8>, true, false, 8), most(traceKernel<true, true, true, kFmWide8>, true, true, 8);
+    most(traceKernel<false, false, false, kFmQuant>, false, false, 4), most(traceKernel<false, true, false, kFmQuant>, false, true, 4);
+    most(traceKernel<true, false, false, kFmQuant>, true, false, 4), most(traceKernel<true, true, false, kFmQuant>, true, true, 4);
+    most(traceKernel<false, false, true, kFmQuant>, false, false, 4), most(traceKernel<false, true, true, kFmQuant>, false, true, 4);
+    most(traceKernel<true, false, true, kFmQuant>, true, false, 4), most(traceKernel<true, true, true, kFmQuant>, true, true, 4);
+    most(traceKernel<false, false, false, kFmPlain, false>, false, false, 4);
+    most(traceKernel<false, false, true, kFmPlain, false>, false, false, 4);
+    most(traceKernel<false, false, false, kFmQuant, false>, false, false, 4);
+    most(traceKernel<false, false, true, kFmQuant, false>, false, false, 4);
+    most(aoTraceKernel<false>, true, true, 4), most(aoTraceKernel<true>, true, true, 4);
+    most(aoTraceKernel<false, kFmWide8>, true, true, 8), most(aoTraceKernel<true, kFmWide8>, true, true, 8);
+    most(aoTraceKernel<false, kFmQuant>, true, true, 4), most(aoTraceKernel<true, kFmQuant>, true, true, 4);
     *sizeBytes = (size_t)threads * gl * sizeof(uint32_t);
     return GRT_SUCCESS;
 }
@@ -924,7 +977,7 @@ grtError grtTraceAmbientOcclusion(grtContext ctx, grtScene scene, const grtRay* 
         : walkFormats(P, true) == kFmQuant ? (count ? aoTraceKernel<true, kFmQuant> : aoTraceKernel<false, kFmQuant>)
                                            : (count ? aoTraceKernel<true> : aoTraceKernel<false>);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t smem = (size_t)bs * traceSmemWords(P.sharedDepth, slotsOf(walkFormats(P, true))) * sizeof(uint32_t);
+    const size_t smem = (size_t)bs * traceSmemWords(true, true, P.sharedDepth, slotsOf(walkFormats(P, true))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
     // scratch after the global stack: the hit count (256 B), the list of hit pixels and
     // their AO frames (48 B each)
@@ -937,7 +990,6 @@ grtError grtTraceAmbientOcclusion(grtContext ctx, grtScene scene, const grtRay* 
     float4* frames = reinterpret_cast<float4*>(static_cast<char*>(extra) + 256 + listBytes);
     uint32_t* counts = reinterpret_cast<uint32_t*>(ao);
     P.counter = nextCounter(c);
-    GRT_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(unsigned long long), s));
     GRT_CUDA(cudaMemsetAsync(listCount, 0, sizeof(uint32_t), s));
     aoCompactKernel<<<ceilDiv(pixelCount, 256), 256, 0, s>>>(P, pixelCount, list, listCount, counts, frames);
     kernel<<<L.blocks, bs, smem, s>>>(P, list, listCount, counts, frames);
@@ -1246,13 +1298,12 @@ static grtError launchShadeForward(Context* c, bool scene, TraceParams& P, const
         : walkFormats(P, scene) == kFmQuant
             ? (scene ? shadeForwardKernel<true, kFmQuant> : shadeForwardKernel<false, kFmQuant>)
             : (scene ? shadeForwardKernel<true> : shadeForwardKernel<false>);
-    const size_t smem = (size_t)bs * traceSmemWords(P.sharedDepth, slotsOf(walkFormats(P, scene))) * sizeof(uint32_t);
+    const size_t smem = (size_t)bs * traceSmemWords(true, scene, P.sharedDepth, slotsOf(walkFormats(P, scene))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
-    L.blocks = std::min<int>(L.blocks, (int)ceilDiv(S.n, bs));
+    L.blocks = traceBlocks(options, P, L, S.n);
     grtError e = bindGlobalStack(c, options, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);
-    GRT_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(unsigned long long), s));
     kernel<<<L.blocks, bs, smem, s>>>(P, S);
     GRT_LAUNCH_CHECK();
     noteLaunches(1);
@@ -1316,7 +1367,6 @@ static grtError shadeBackward(grtContext ctx, grtScene scene, grtGeometry geom, 
     L.blocks = std::min(L.blocks, 8 * smCount(c));
     L.blocks = std::min<int>(L.blocks, (int)ceilDiv(n, bs));
     P.counter = nextCounter(c);
-    GRT_CUDA(cudaMemsetAsync(P.counter, 0, sizeof(unsigned long long), s));
     kernel<<<L.blocks, bs, smem, s>>>(P, S, priv ? nv : 0u);
     GRT_LAUNCH_CHECK();
     noteLaunches(1);
