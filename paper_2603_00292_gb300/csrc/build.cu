@@ -482,17 +482,14 @@ static grtError launchNodeFormats(const BvhObject* o, cudaStream_t s) {
 
 // ======================================================================= small builds
 // Up to kSmallBuild primitives (kSmallScene instances) a build runs in one block of
-// kSmallBuildThreads threads, as one launch, instead of a dozen grid-wide launches whose
-// cost is their own latency at this size. The thresholds are where the measured times
-// cross (one block against the graph of grid launches, 30-bit codes): a 1,280-triangle
-// icosphere 0.070 vs 0.080 ms, 2,048 triangles 0.093 vs 0.083 ms, 4,050 triangles 0.19
-// vs 0.095 ms; a top level of 4,000 instances 0.61 vs 0.15 ms (its FP64 instance setup
-// runs on one SM). Up to kSharedFitMax primitives the block keeps the whole build on
-// chip (bitonicSortShared, fitLeafShared).
-#ifndef GRT_SMALL_BUILD
-#define GRT_SMALL_BUILD 2048
-#endif
-constexpr uint32_t kSmallBuild = GRT_SMALL_BUILD;
+// kSmallBuildThreads threads, as one launch, instead of a graph of some nine grid-wide
+// launches whose cost is their own latency at this size. The threshold is where the measured
+// times cross (us, one block against the graph, 30-bit codes): 512 triangles 35 / 35, 768 43 /
+// 41, 1,024 49 / 43, 1,280 67 / 45, 2,048 80 / 45; the first build of a geometry, which also
+// captures its graph, 69 / 100 at 1,024, 83 / 105 at 1,280 and 99 / 103 at 2,048. A top level of 4,000 instances
+// took 0.61 against 0.15 ms (its FP64 instance setup runs on one SM). Up to kSharedFitMax
+// primitives the block keeps the whole build on chip (bitonicSortShared, fitLeafShared).
+constexpr uint32_t kSmallBuild = 1024;
 constexpr uint32_t kSmallScene = 1024;
 #ifndef GRT_SMALL_BUILD_THREADS
 #define GRT_SMALL_BUILD_THREADS 1024
