@@ -642,8 +642,9 @@ typedef struct grtBatchOptions {
     float compactThreshold;     /* refill a warp when <= this fraction of lanes hold a ray [0.75] */
     uint32_t smallScenePrims;   /* scenes up to this many triangles are built by one block [8192] */
     uint32_t sortChunkTiles;    /* radix tiles (blockSize x 8 keys) per sort work item [8] */
-    uint32_t buildChunk;        /* primitives per prep / emission / fit work item [16384] */
-    uint32_t traceChunk;        /* rays per trace work item [16384] */
+    uint32_t buildChunk;        /* primitives per prep / emission / fit work item [16384, or fewer,
+                                   down to 1024, in a batch too small to give every block items] */
+    uint32_t traceChunk;        /* rays per trace work item [16384, or fewer, down to 512, likewise] */
     uint32_t sceneGroup;        /* scenes per scheduling group, largest first: a group's builds, then its
                                    traces [32] */
     uint32_t waitLimitMs;       /* a work item's wait for another expires after this long [2000] */
