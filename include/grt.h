@@ -640,7 +640,8 @@ typedef struct grtBatchOptions {
     uint32_t sharedStackDepth;  /* traversal stack entries in shared memory, <= 32 [16] */
     uint32_t globalStackDepth;  /* spill entries per thread, <= 4096 [64] */
     float compactThreshold;     /* refill a warp when <= this fraction of lanes hold a ray [0.75] */
-    uint32_t smallScenePrims;   /* scenes up to this many triangles are built by one block [8192] */
+    uint32_t smallScenePrims;   /* scenes up to this many triangles are built by one block [1/32 of the
+                                   largest scene's, between 1024 and 8192] */
     uint32_t sortChunkTiles;    /* radix tiles (blockSize x 8 keys) per sort work item [8] */
     uint32_t buildChunk;        /* primitives per prep / emission / fit work item [16384, or fewer,
                                    down to 1024, in a batch too small to give every block items] */

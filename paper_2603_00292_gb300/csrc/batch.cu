@@ -386,9 +386,8 @@ static grtError resolveBatchOptions(const grtBatchOptions* o, grtBatchOptions* r
     if (!d.sharedStackDepth) d.sharedStackDepth = 16;
     if (!d.globalStackDepth) d.globalStackDepth = 64;
     if (!(d.compactThreshold > 0.f)) d.compactThreshold = 0.75f;
-    if (!d.smallScenePrims) d.smallScenePrims = 8192;
     if (!d.sortChunkTiles) d.sortChunkTiles = 8;
-    // buildChunk and traceChunk: 0 until the batch's size is known (chunkFor)
+    // smallScenePrims, buildChunk and traceChunk: 0 until the batch's size is known
     if (!d.sceneGroup) d.sceneGroup = 32;
     if (!d.waitLimitMs) d.waitLimitMs = 2000;
     if (d.blockSize != 64 && d.blockSize != 128 && d.blockSize != 256) return GRT_ERROR_INVALID_PARAMETER;
@@ -449,12 +448,18 @@ grtError grtCreateBatch(grtContext ctx, const grtBatchScene* scenes, uint32_t sc
         perSm < 1)
         perSm = 1;
     uint64_t totalRays = 0, totalPrims = 0;
+    uint32_t mostPrims = 0;
     for (uint32_t i = 0; i < sceneCount; ++i) {
         totalRays += scenes[i].rayCount;
         uint32_t n = 0;
-        if (validateGeometryInput(&scenes[i].input, &n) == GRT_SUCCESS) totalPrims += n;
+        if (validateGeometryInput(&scenes[i].input, &n) == GRT_SUCCESS) totalPrims += n, mostPrims = std::max(mostPrims, n);
     }
     const uint32_t gridBlocks = (uint32_t)perSm * (uint32_t)smCount(c);
+    // One block builds 8,192 primitives in 2.4 ms, which is fine beside the builds and rays of
+    // much larger scenes and is what the launch waits for otherwise: up to 1/32 of the largest
+    // scene (23 scenes of up to 46,000 triangles 2.52 -> 1.91 ms, 160 of up to 20,000 4.22 ->
+    // 2.90 with 1,024; 24 of up to 266,000 stay at 8,192, 10.9 against 11.1 with 1,024).
+    if (!opt.smallScenePrims) opt.smallScenePrims = std::min(8192u, std::max(1024u, mostPrims / 32));
     if (!opt.buildChunk) opt.buildChunk = chunkFor(totalPrims, gridBlocks, 1024);
     if (!opt.traceChunk) opt.traceChunk = chunkFor(totalRays, gridBlocks, 512);
     const uint32_t chunkKeys = opt.sortChunkTiles * bs * kBlockSortItems;
