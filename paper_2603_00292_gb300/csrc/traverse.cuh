@@ -181,17 +181,22 @@ __device__ __forceinline__ float3 slabReciprocal(float3 d) {
     return r;
 }
 
+//
+// A zero component's reciprocal is finite here (slabReciprocal), so a ray that lies in a plane
+// of the box itself would get distance 0 for it, where the difference form's 0 inf drops it.
+// kPlane |id| on either side, nothing at ordinary reciprocals, puts such a plane past every t.
+constexpr float kPlane = 1e-20f;
 template <bool FUSED>
 __device__ __forceinline__ float slabNear(float o, float id) {
     if constexpr (!FUSED) return o;
     const float q = o * id;  // a factor, not a sum: an infinite product stays one
-    return -q * (q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps);
+    return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -kPlane * fabsf(id));
 }
 template <bool FUSED>
 __device__ __forceinline__ float slabFar(float o, float id) {
     if constexpr (!FUSED) return o;
     const float q = o * id;
-    return -q * (q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps);
+    return fmaf(-q, q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps, kPlane * fabsf(id));
 }
 template <bool FUSED>
 __device__ __forceinline__ float slabAt(float p, float id, float c) {

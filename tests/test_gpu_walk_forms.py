@@ -118,3 +118,36 @@ def test_rays_that_are_not_finite_miss(gpu, fmt, two_level):
     if scene:
         scene.close()
     g.close()
+
+
+@pytest.mark.parametrize("fmt", list(FORMATS))
+@pytest.mark.parametrize("two_level", [False, True])
+def test_rays_in_the_planes_of_boxes_hit_inclusive_edges(gpu, fmt, two_level):
+    """Rays straight down on the vertices and edges of a flat grid whose far sides lie at 0: they
+    lie in the planes of the boxes, and edges belong to their triangles."""
+    m = scenegen.terrain(8, 0.0)
+    v = m.vertices.copy()
+    v[:, [0, 2]] -= 1.0  # [-2, 0]^2, multiples of 1/4
+    g = Geometry(gpu, vertices=device_tensor(v), indices=device_tensor(m.indices), build_flags=FORMATS[fmt]).build()
+    k = np.concatenate([np.arange(9) / 4.0 - 2.0, [-0.0]]).astype(np.float32)
+    x, z = (a.ravel() for a in np.meshgrid(k, np.concatenate([k, k[:8] + 0.125])))
+    rays = np.zeros((2 * x.size, 8), np.float32)
+    rays[:, 0], rays[:, 2] = np.tile(x, 2), np.tile(z, 2)
+    rays[:, 1] = 1.0
+    rays[:, 5] = -1.0
+    rays[x.size:, [4, 6]] = -0.0
+    rays[:, 7] = np.inf
+    scene = None
+    if two_level:
+        f = np.array([[0, 0, 0, 1, 1, 1, 1, 0, 0, 0]], np.float32)
+        scene = Scene(gpu, [g.handle], device_tensor(f), build_flags=FORMATS[fmt] if fmt == "wide8" else 0).build()
+    args = dict(scene=scene.handle) if scene else dict(geom=g.handle)
+    r = device_tensor(rays)
+    for any_hit in (False, True):
+        _, prim, t, _, _ = hits_to_numpy(_trace(gpu, r, any_hit=any_hit, **args))
+        assert (prim != NONE).all() and np.all(np.abs(t - 1.0) <= 1e-5)
+    big = r.repeat(-(-(1 << 20) // r.shape[0]), 1)[:1 << 20].contiguous()  # the per-ray form
+    assert (hits_to_numpy(_trace(gpu, big, **args))[1] != NONE).all()
+    if scene:
+        scene.close()
+    g.close()
