@@ -627,20 +627,26 @@ static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int thre
         *extra = p;
         return e;
     }
-    grtError e = contextScratch(c, std::max<size_t>(need + extraBytes, 256), &p);
+    // at the usual depths the area is made for the largest grid at once, so that no later
+    // trace of another kind or size grows it (growing waits for the device)
+    const size_t most = P.globalDepth <= 64 ? (size_t)smCount(c) * 2048 * P.globalDepth * sizeof(uint32_t) : 0;
+    grtError e = contextScratch(c, std::max<size_t>(std::max(need, most) + extraBytes, 256), &p);
     P.globalStack = (uint32_t*)p;
     if (extraBytes) *extra = static_cast<char*>(p) + need;
     return e;
 }
 
 // Blocks of a trace of n items: a warp takes one at least (itemLanes). A caller's own stack
-// buffer that holds a block per blockSize items, but not these, keeps the grid to what it
-// holds.
-static int traceBlocks(const grtTraceOptions* opt, const TraceParams& P, LaunchShape L, uint32_t n) {
+// buffer keeps the grid to what it holds, down to a block per blockSize items and at most
+// 640 threads an SM for any hits in one geometry, 512 for the others, below which it is
+// refused.
+static int traceBlocks(Context* c, const grtTraceOptions* opt, const TraceParams& P, LaunchShape L, uint32_t n,
+                       bool any, bool scene) {
     const int spread = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize / 32));
     if (!opt || !opt->globalStack || P.globalDepth == 0) return spread;
     const size_t fits = (opt->globalStackBytes & ~(size_t)255) / ((size_t)L.blockSize * P.globalDepth * sizeof(uint32_t));
-    const int least = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize));
+    const int sms = smCount(c) * ((any && !scene ? 640 : 512) / L.blockSize);
+    const int least = std::min(std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize)), sms);
     return std::max(least, (int)std::min<size_t>(fits, (size_t)spread));
 }
 
@@ -700,7 +706,7 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
     cudaStream_t s = (cudaStream_t)stream;
     const size_t smem = (size_t)bs * traceSmemWords(ANY, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
-    L.blocks = traceBlocks(opt, P, L, n);
+    L.blocks = traceBlocks(c, opt, P, L, n, ANY, isScene);
     e = bindGlobalStack(c, opt, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);
@@ -1300,7 +1306,7 @@ static grtError launchShadeForward(Context* c, bool scene, TraceParams& P, const
             : (scene ? shadeForwardKernel<true> : shadeForwardKernel<false>);
     const size_t smem = (size_t)bs * traceSmemWords(true, scene, P.sharedDepth, slotsOf(walkFormats(P, scene))) * sizeof(uint32_t);
     LaunchShape L = persistentShape(c, kernel, bs, smem);
-    L.blocks = traceBlocks(options, P, L, S.n);
+    L.blocks = traceBlocks(c, options, P, L, S.n, true, scene);
     grtError e = bindGlobalStack(c, options, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);

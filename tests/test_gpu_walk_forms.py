@@ -151,3 +151,26 @@ def test_rays_in_the_planes_of_boxes_hit_inclusive_edges(gpu, fmt, two_level):
     if scene:
         scene.close()
     g.close()
+
+
+@pytest.mark.parametrize("any_hit", [False, True])
+@pytest.mark.parametrize("n", [5000, 50_000, 1 << 20])
+def test_a_callers_stack_buffer_bounds_the_grid(gpu, n, any_hit):
+    _, g = _terrain(gpu, 0)
+    rays = new_rays(n)
+    grt.grtGenerateUniformRays(gpu.handle, [-1, -1, -1], [1, 1, 1], 9, n, rays)
+    whole = _trace(gpu, rays, geom=g.handle, any_hit=any_hit)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    blocks = min(-(-n // 128), sms * (5 if any_hit else 4))
+    f = grt.grtTraceAnyHit if any_hit else grt.grtTraceClosest
+    for size, accepted in ((blocks * 128 * 64 * 4, True), (blocks * 128 * 64 * 4 - 256, False)):
+        stack = torch.empty(size, dtype=torch.uint8, device="cuda")
+        o = grt.trace_options(global_stack=stack, global_stack_bytes=size)
+        hits = new_hits(n)
+        if accepted:
+            f(gpu.handle, None, g.handle, rays, n, hits, None, o)
+            assert torch.equal(hits, whole)
+        else:
+            with pytest.raises(grt.GrtError):
+                f(gpu.handle, None, g.handle, rays, n, hits, None, o)
+    g.close()
