@@ -89,8 +89,8 @@ __device__ __forceinline__ Box3 emitLeaf(const FitParams& P, uint32_t k) {
     }
 }
 
-// Box of leaf k, written by another block of this launch: a whole triangle's comes from its
-// leaf record in one step, others from the input.
+// Box of leaf k, written by an earlier launch: a whole triangle's comes from its leaf record
+// in one step, others from the input.
 template <int KIND>
 __device__ __forceinline__ Box3 leafBox(const FitParams& P, uint32_t k) {
     if (KIND == 0 && P.src.kind == 0) {
@@ -101,38 +101,19 @@ __device__ __forceinline__ Box3 leafBox(const FitParams& P, uint32_t k) {
     return emitLeaf<KIND, false>(P, k);
 }
 
-__device__ __forceinline__ Box3 emptyBox() {
-    return Box3{make_float3(INFINITY, INFINITY, INFINITY), make_float3(-INFINITY, -INFINITY, -INFINITY)};
-}
 __device__ __forceinline__ Box3 unionBox(const Box3& a, const Box3& b) {
     return Box3{make_float3(fminf(a.lo.x, b.lo.x), fminf(a.lo.y, b.lo.y), fminf(a.lo.z, b.lo.z)),
                 make_float3(fmaxf(a.hi.x, b.hi.x), fmaxf(a.hi.y, b.hi.y), fmaxf(a.hi.z, b.hi.z))};
 }
 
-// A subtree on its way up: its child word, leaf range, and the two slots it takes in its
-// parent's 4-wide node (its children, or itself and an empty slot).
-struct Subtree {
-    uint32_t self, l, r;
-    Box3 s0, s1;
-    uint32_t w0, w1;
-};
-
-// The subtree of child word w over [l, r], its node or leaf written by another block.
+// Box of the subtree of child word w, its node or leaf written by an earlier launch.
 template <int KIND>
-__device__ __forceinline__ Subtree loadSubtree(const FitParams& P, uint32_t w, uint32_t l, uint32_t r) {
-    Subtree u;
-    u.self = w, u.l = l, u.r = r;
-    if (w & kLeafBit) {
-        u.s0 = leafBox<KIND>(P, w & ~kLeafBit), u.s1 = emptyBox();
-        u.w0 = w, u.w1 = kInvalid;
-    } else {
-        const float4* N = P.nodes + 4 * (size_t)w;
-        const float4 x = __ldcg(N), y = __ldcg(N + 1), z = __ldcg(N + 2), c = __ldcg(N + 3);
-        u.s0 = Box3{make_float3(x.x, y.x, z.x), make_float3(x.y, y.y, z.y)};
-        u.s1 = Box3{make_float3(x.z, y.z, z.z), make_float3(x.w, y.w, z.w)};
-        u.w0 = __float_as_uint(c.x), u.w1 = __float_as_uint(c.y);
-    }
-    return u;
+__device__ __forceinline__ Box3 subtreeBox(const FitParams& P, uint32_t w) {
+    if (w & kLeafBit) return leafBox<KIND>(P, w & ~kLeafBit);
+    const float4* N = P.nodes + 4 * (size_t)w;
+    const float4 x = __ldcg(N), y = __ldcg(N + 1), z = __ldcg(N + 2);
+    return Box3{make_float3(fminf(x.x, x.z), fminf(y.x, y.z), fminf(z.x, z.z)),
+                make_float3(fmaxf(x.y, x.w), fmaxf(y.y, y.w), fmaxf(z.y, z.w))};
 }
 
 // A block's nodes in shared memory, numbered from its first leaf: node p as p - first leaf
@@ -320,8 +301,7 @@ __global__ void __launch_bounds__(kTopThreads) emitTopKernel(EmitParams E, const
         uint32_t list = 0;
         for (uint32_t j = 1; j < kTopFan; ++j) list = i >= S.first[j] ? j : list;
         const uint4 top = in.tops[(size_t)(list0 + list) * kTopMax + (i - S.first[list])];
-        const Subtree u = loadSubtree<KIND>(P, top.x, top.y, top.z);
-        const Box3 b = unionBox(u.s0, u.s1);
+        const Box3 b = subtreeBox<KIND>(P, top.x);
         const uint32_t id = kTopCap + i;
         S.box[0][id] = b.lo.x, S.box[2][id] = b.lo.y, S.box[4][id] = b.lo.z;
         S.box[1][id] = b.hi.x, S.box[3][id] = b.hi.y, S.box[5][id] = b.hi.z;
