@@ -127,6 +127,7 @@ __device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a
 __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
     return make_float3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
+__device__ __forceinline__ float3 abs3(float3 a) { return make_float3(fabsf(a.x), fabsf(a.y), fabsf(a.z)); }
 __device__ __forceinline__ float norm1(float3 a) { return fabsf(a.x) + fabsf(a.y) + fabsf(a.z); }
 __device__ __forceinline__ float3 normalize3(float3 a) {
     const float l = sqrtf(dot3(a, a));
@@ -162,21 +163,29 @@ struct Level {
 // and a difference needs no care with zero directions.
 __host__ __device__ constexpr bool fusedSlab(bool any, bool scene) { return any || !scene; }
 
-// Reciprocal direction for the slab tests. Fused, a zero component's must be finite: an
-// infinite one makes fma(p, inf, -o inf) a NaN and the axis cull nothing. Where some
-// component is of ordinary size (its reciprocal below 2^66), reciprocals are therefore kept
-// within 2^106: the planes of a smaller component then still lie past every t the ray can
-// have, on the right side. (Clamped without a branch: a test for infinities and a fix-up
-// cost one instruction in eight of a scene's closest hits.)
+// Reciprocal direction for the slab tests; a bounds the origins of the level per axis.
+// Fused, neither a reciprocal nor its product with the origin may be infinite: fma(p, inf,
+// -o inf) is a NaN at best, and with an infinite product alone every plane lies on one side.
+// Reciprocals are therefore kept within the power of two that keeps the product below 2^126;
+// the planes of a smaller component then still lie past every t the ray can have, on the
+// right side. The ray's reach bounds that t: for directions shorter than 2^-38, whose rays
+// reach too far, larger reciprocals become infinite instead, and such an axis culls little or
+// nothing. (Without a branch: a test for infinities and a fix-up cost one instruction in eight
+// of a scene's closest hits.)
+__device__ __forceinline__ float slabCap(float a) {
+    return __uint_as_float(0xBD800000u - (__float_as_uint(fmaxf(a, 1.f)) & 0x7F800000u));  // 2^(125 - exponent of a)
+}
+__device__ __forceinline__ float slabClamp(float r, float cap, bool reaches) {
+    return fabsf(r) > cap ? copysignf(reaches ? cap : INFINITY, r) : r;
+}
 template <bool FUSED>
-__device__ __forceinline__ float3 slabReciprocal(float3 d) {
+__device__ __forceinline__ float3 slabReciprocal(float3 d, float3 a) {
     float3 r = make_float3(__frcp_rn(d.x), __frcp_rn(d.y), __frcp_rn(d.z));
     if constexpr (FUSED) {
-        const float least = fminf(fminf(fabsf(r.x), fabsf(r.y)), fabsf(r.z));
-        const float cap = least < 7.3786976e19f ? 8.1129638e31f : INFINITY;
-        r.x = fminf(fmaxf(r.x, -cap), cap);
-        r.y = fminf(fmaxf(r.y, -cap), cap);
-        r.z = fminf(fmaxf(r.z, -cap), cap);
+        const bool reaches = fminf(fminf(fabsf(r.x), fabsf(r.y)), fabsf(r.z)) < 2.74877907e11f;  // 2^38
+        r.x = slabClamp(r.x, slabCap(a.x), reaches);
+        r.y = slabClamp(r.y, slabCap(a.y), reaches);
+        r.z = slabClamp(r.z, slabCap(a.z), reaches);
     }
     return r;
 }
@@ -189,7 +198,7 @@ constexpr float kPlane = 1e-20f;
 template <bool FUSED>
 __device__ __forceinline__ float slabNear(float o, float id) {
     if constexpr (!FUSED) return o;
-    const float q = o * id;  // a factor, not a sum: an infinite product stays one
+    const float q = o * id;  // infinite only with o, and then still so after the factor
     return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -kPlane * fabsf(id));
 }
 template <bool FUSED>
@@ -663,7 +672,6 @@ __device__ __forceinline__ void instanceLevel(Level& L, const InstanceRecord* R,
     }
     L.o = make_float3(o[0], o[1], o[2]);
     L.d = make_float3(d[0], d[1], d[2]);
-    L.id = slabReciprocal<FUSED>(L.d);
     L.dl1 = norm1(L.d);
     L.tOff = te;
     // final rounding (u) plus the float-float evaluation's own error (tens of u^2
@@ -673,6 +681,7 @@ __device__ __forceinline__ void instanceLevel(Level& L, const InstanceRecord* R,
     L.dD = 6.f * kEps * sd;
     const float span = fmaxf(fabsf(texit - te), fabsf(tmin - te)) * (1.f + 4.f * kEps);
     const float slack = L.dO + span * L.dD + 2.f * kEps * so;
+    L.id = slabReciprocal<FUSED>(L.d, make_float3(fabsf(o[0]) + slack, fabsf(o[1]) + slack, fabsf(o[2]) + slack));
     const float3 sg = make_float3(copysignf(slack, L.id.x), copysignf(slack, L.id.y), copysignf(slack, L.id.z));
     L.cn = make_float3(slabNear<FUSED>(L.o.x + sg.x, L.id.x), slabNear<FUSED>(L.o.y + sg.y, L.id.y), slabNear<FUSED>(L.o.z + sg.z, L.id.z));
     L.cf = make_float3(slabFar<FUSED>(L.o.x - sg.x, L.id.x), slabFar<FUSED>(L.o.y - sg.y, L.id.y), slabFar<FUSED>(L.o.z - sg.z, L.id.z));
@@ -794,7 +803,7 @@ __device__ __forceinline__ void beginRay(const TraceParams& P, Stack& st, RaySta
     s.wd = wd;
     s.tmin = tmin;
     s.tmax = tmax;
-    s.wid = slabReciprocal<FUSED>(wd);
+    s.wid = slabReciprocal<FUSED>(wd, abs3(wo));
     exactLevel<FUSED>(s.L, wo, wd, s.wid);
     s.nodes = P.target.nodes;
     s.fmt = P.target.fmt;
