@@ -172,6 +172,7 @@ __host__ __device__ constexpr bool fusedSlab(bool any, bool scene) { return any 
 // reach too far, larger reciprocals become infinite instead, and such an axis culls little or
 // nothing. (Without a branch: a test for infinities and a fix-up cost one instruction in eight
 // of a scene's closest hits.)
+constexpr float kSlabReach = 2.74877907e11f;  // 2^38
 __device__ __forceinline__ float slabCap(float a) {
     return __uint_as_float(0xBD800000u - (__float_as_uint(fmaxf(a, 1.f)) & 0x7F800000u));  // 2^(125 - exponent of a)
 }
@@ -182,7 +183,7 @@ template <bool FUSED>
 __device__ __forceinline__ float3 slabReciprocal(float3 d, float3 a) {
     float3 r = make_float3(__frcp_rn(d.x), __frcp_rn(d.y), __frcp_rn(d.z));
     if constexpr (FUSED) {
-        const bool reaches = fminf(fminf(fabsf(r.x), fabsf(r.y)), fabsf(r.z)) < 2.74877907e11f;  // 2^38
+        const bool reaches = fminf(fminf(fabsf(r.x), fabsf(r.y)), fabsf(r.z)) < kSlabReach;
         r.x = slabClamp(r.x, slabCap(a.x), reaches);
         r.y = slabClamp(r.y, slabCap(a.y), reaches);
         r.z = slabClamp(r.z, slabCap(a.z), reaches);
@@ -190,26 +191,39 @@ __device__ __forceinline__ float3 slabReciprocal(float3 d, float3 a) {
     return r;
 }
 
-//
-// A zero component's reciprocal is finite here (slabReciprocal), so a ray that lies in a plane
-// of the box itself would get distance 0 for it, where the difference form's 0 inf drops it.
-// kPlane |id| on either side, nothing at ordinary reciprocals, puts such a plane past every t.
-constexpr float kPlane = 1e-20f;
-template <bool FUSED>
-__device__ __forceinline__ float slabNear(float o, float id) {
-    if constexpr (!FUSED) return o;
-    const float q = o * id;  // infinite only with o, and then still so after the factor
-    return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -kPlane * fabsf(id));
+// A clamped reciprocal is finite, so a ray that lies in a plane of the box itself gets distance
+// 0 for it where the difference form's 0 inf drops it. Planes within `width` of the origin are
+// therefore moved to either side by width |id|. At the largest reciprocal, 2^125, that is 2^63
+// times the least reciprocal: past any t at which the ray is still within 2^63 of the box, whose
+// squares are the last a float32 holds. At ordinary reciprocals it is nothing. (Farther out than
+// 1, where reciprocals are kept smaller, the roundings below are 2^102.)
+__device__ __forceinline__ float slabWidth(float3 id) {
+    const float least = fminf(fminf(fabsf(id.x), fabsf(id.y)), fabsf(id.z));
+    return least < kSlabReach ? least * 2.16840434e-19f : 0.f;  // 2^-62
 }
 template <bool FUSED>
-__device__ __forceinline__ float slabFar(float o, float id) {
+__device__ __forceinline__ float slabNear(float o, float id, float width) {
+    if constexpr (!FUSED) return o;
+    const float q = o * id;  // infinite only with o, and then still so after the factor
+    return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -width * fabsf(id));
+}
+template <bool FUSED>
+__device__ __forceinline__ float slabFar(float o, float id, float width) {
     if constexpr (!FUSED) return o;
     const float q = o * id;
-    return fmaf(-q, q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps, kPlane * fabsf(id));
+    return fmaf(-q, q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps, width * fabsf(id));
 }
 template <bool FUSED>
 __device__ __forceinline__ float slabAt(float p, float id, float c) {
     return FUSED ? fmaf(p, id, c) : (p - c) * id;
+}
+
+// Terms of L's slab distances for origins n of the near and f of the far planes (L.id set).
+template <bool FUSED>
+__device__ __forceinline__ void setSlabs(Level& L, float3 n, float3 f) {
+    const float w = FUSED ? slabWidth(L.id) : 0.f;
+    L.cn = make_float3(slabNear<FUSED>(n.x, L.id.x, w), slabNear<FUSED>(n.y, L.id.y, w), slabNear<FUSED>(n.z, L.id.z, w));
+    L.cf = make_float3(slabFar<FUSED>(f.x, L.id.x, w), slabFar<FUSED>(f.y, L.id.y, w), slabFar<FUSED>(f.z, L.id.z, w));
 }
 
 template <bool FUSED>
@@ -217,8 +231,7 @@ __device__ __forceinline__ void exactLevel(Level& L, float3 o, float3 d, float3 
     L.o = o;
     L.d = d;
     L.id = id;
-    L.cn = make_float3(slabNear<FUSED>(o.x, id.x), slabNear<FUSED>(o.y, id.y), slabNear<FUSED>(o.z, id.z));
-    L.cf = make_float3(slabFar<FUSED>(o.x, id.x), slabFar<FUSED>(o.y, id.y), slabFar<FUSED>(o.z, id.z));
+    setSlabs<FUSED>(L, o, o);
     L.dO = 0.f;
     L.dD = 0.f;
     L.dl1 = norm1(d);
@@ -653,11 +666,12 @@ __device__ __forceinline__ void instanceLevel(Level& L, const InstanceRecord* R,
                                               float3 wd, float3 wid, float tmin, float lim) {
     const float4 m[3] = {R->inv[0], R->inv[1], R->inv[2]};
     const float4 blo = R->worldLo, bhi = R->worldHi;
-    // entry and exit parameters of the world box (exact world ray, conservative)
+    // entry and exit parameters of the world box (exact world ray, conservative); L is still
+    // the world's level, whose far distances a ray in a plane of the box passes
     const bool px = wid.x >= 0.f, py = wid.y >= 0.f, pz = wid.z >= 0.f;
-    const float nx = ((px ? blo.x : bhi.x) - wo.x) * wid.x, fx = ((px ? bhi.x : blo.x) - wo.x) * wid.x;
-    const float ny = ((py ? blo.y : bhi.y) - wo.y) * wid.y, fy = ((py ? bhi.y : blo.y) - wo.y) * wid.y;
-    const float nz = ((pz ? blo.z : bhi.z) - wo.z) * wid.z, fz = ((pz ? bhi.z : blo.z) - wo.z) * wid.z;
+    const float nx = ((px ? blo.x : bhi.x) - wo.x) * wid.x, fx = slabAt<FUSED>(px ? bhi.x : blo.x, wid.x, L.cf.x);
+    const float ny = ((py ? blo.y : bhi.y) - wo.y) * wid.y, fy = slabAt<FUSED>(py ? bhi.y : blo.y, wid.y, L.cf.y);
+    const float nz = ((pz ? blo.z : bhi.z) - wo.z) * wid.z, fz = slabAt<FUSED>(pz ? bhi.z : blo.z, wid.z, L.cf.z);
     const float tentry = fmaxf(fmaxf(nx, ny), fmaxf(nz, tmin));
     const float texit = fminf(fminf(fx, fy), fminf(fz, lim)) * kFarScale;
     const float te = (tentry < texit && tentry < INFINITY) ? tentry : tmin;  // any finite shift is exact enough
@@ -683,8 +697,7 @@ __device__ __forceinline__ void instanceLevel(Level& L, const InstanceRecord* R,
     const float slack = L.dO + span * L.dD + 2.f * kEps * so;
     L.id = slabReciprocal<FUSED>(L.d, make_float3(fabsf(o[0]) + slack, fabsf(o[1]) + slack, fabsf(o[2]) + slack));
     const float3 sg = make_float3(copysignf(slack, L.id.x), copysignf(slack, L.id.y), copysignf(slack, L.id.z));
-    L.cn = make_float3(slabNear<FUSED>(L.o.x + sg.x, L.id.x), slabNear<FUSED>(L.o.y + sg.y, L.id.y), slabNear<FUSED>(L.o.z + sg.z, L.id.z));
-    L.cf = make_float3(slabFar<FUSED>(L.o.x - sg.x, L.id.x), slabFar<FUSED>(L.o.y - sg.y, L.id.y), slabFar<FUSED>(L.o.z - sg.z, L.id.z));
+    setSlabs<FUSED>(L, L.o + sg, L.o - sg);
 }
 
 struct Stack {

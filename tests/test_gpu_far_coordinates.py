@@ -1,6 +1,7 @@
 """Rays with zero direction components far from the origin of coordinates, where the product
 of the origin and a reciprocal direction leaves the range of a float32 (from 2^22 on at a
-reciprocal of 2^106), compared with the oracle."""
+reciprocal of 2^106), compared with the oracle; and rays in the planes of boxes whatever the
+length of their direction."""
 import ctypes
 
 import numpy as np
@@ -117,4 +118,37 @@ def test_far_axis_aligned_rays_in_a_batch_and_a_user_kernel(gpu, user_lib, shift
         else:
             compare_closest(got, ref, S, rays, extent=extent).check()
     b.close()
+    g.close()
+
+
+@pytest.mark.parametrize("fmt", list(FORMATS))
+@pytest.mark.parametrize("two_level", [False, True])
+@pytest.mark.parametrize("length, height", [(1.0, 1e9), (1e-4, 1.0), (1e-8, 1e4), (1e-12, 1.0), (1e-12, 1e8), (1e-20, 1e3)])
+def test_rays_in_box_planes_hit_with_directions_of_any_length(gpu, two_level, fmt, length, height):
+    """Straight down on the vertices and edges of a flat grid in [-2, 0]^2: boxes have planes at 0,
+    in which rays lie; edges belong to their triangles."""
+    m = scenegen.terrain(8, 0.0)
+    v = m.vertices.copy()
+    v[:, [0, 2]] -= 1.0
+    g = Geometry(gpu, vertices=device_tensor(v), indices=device_tensor(m.indices), build_flags=FORMATS[fmt]).build()
+    k = np.concatenate([np.arange(9) / 4.0 - 2.0, [-0.0]]).astype(np.float32)
+    x, z = (a.ravel() for a in np.meshgrid(k, np.concatenate([k, k[:8] + 0.125])))
+    rays = np.zeros((2 * x.size, 8), np.float32)
+    rays[:, 0], rays[:, 2] = np.tile(x, 2), np.tile(z, 2)
+    rays[:, 1] = height
+    rays[:, 5] = -length
+    rays[x.size:, [4, 6]] = -0.0
+    rays[:, 7] = np.inf
+    scene = None
+    if two_level:
+        f = np.array([[0, 0, 0, 1, 1, 1, 1, 0, 0, 0]], np.float32)
+        scene = Scene(gpu, [g.handle], device_tensor(f), build_flags=FORMATS[fmt] if fmt == "wide8" else 0).build()
+    args = dict(scene=scene.handle) if scene else dict(geom=g.handle)
+    r = device_tensor(rays)
+    t = np.float64(np.float32(height)) / np.float64(np.float32(length))
+    for any_hit in (False, True):
+        got = _trace(gpu, r, any_hit=any_hit, **args)
+        assert (got[1] != NONE).all() and np.all(np.abs(got[2] - t) <= 1e-5 * t)
+    if scene:
+        scene.close()
     g.close()
