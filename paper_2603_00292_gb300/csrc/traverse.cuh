@@ -737,6 +737,10 @@ struct Stack {
     }
 };
 
+// Whether a stack entry at distance t (its low bits cut off, towards 0) lies behind the limit
+// hi. Below 0 the cut brings the entry closer to the limit, so none is dropped there.
+__device__ __forceinline__ bool behindHit(float t, float hi) { return t > fmaxf(hi, 0.f) * kFarScale; }
+
 // Per-ray work counts (only with COUNT): nodes, triangles, customs, instances, FP64 tests.
 struct Visits {
     uint32_t nodes = 0, tris = 0, customs = 0, insts = 0, fp64 = 0;
@@ -1148,7 +1152,7 @@ __device__ __forceinline__ bool stepRay(const TraceParams& P, Stack& st, RayStat
         if constexpr (AT) {
             float t;
             s.next = st.popAt(t);
-            if (t > s.hi * kFarScale) {  // behind a hit found since it was put there
+            if (behindHit(t, s.hi)) {  // behind a hit found since it was put there
                 s.next = kNone;
                 return false;
             }
@@ -1570,7 +1574,7 @@ __device__ __forceinline__ uint32_t nextState(const TraceParams& P, Stack& st, R
         if constexpr (keepsDistances(ANY, SCENE, W)) {
             float t;
             const uint32_t x = st.popAt(t);
-            s.next = t > s.hi * kFarScale ? kNone : x;
+            s.next = behindHit(t, s.hi) ? kNone : x;
         } else {
             const uint32_t x = st.pop();
             if (SCENE && x == kSentinel) {
