@@ -2,7 +2,10 @@
 // (camera, ambient occlusion) and their host entry points. The traversal itself is in
 // traverse.cuh.
 #include <algorithm>
+#include <map>
 #include <mutex>
+#include <set>
+#include <tuple>
 #include <unordered_map>
 
 #include <cmath>
@@ -522,29 +525,32 @@ struct LaunchShape {
     int blocks;
 };
 
+// The most shared memory a walk can ask for (blocks of 256, 32 shared stack entries).
+constexpr size_t kMostTraceSmem =
+    256 * std::max(traceSmemWords(false, false, 32, 4), traceSmemWords(false, false, 32, 8)) * sizeof(uint32_t);
+
+// Blocks of the persistent grid of `kernel`. Above 48 KB (deep stacks in large blocks) a kernel
+// has to opt in, per device: once, to the most that any call asks of it, so that no later call
+// lowers what another one's cached shape relies on.
 template <class K>
-static LaunchShape persistentShape(Context* c, K kernel, int blockSize, size_t smem) {
+static grtError persistentShape(Context* c, K kernel, int blockSize, size_t smem, LaunchShape* out,
+                                size_t mostSmem = kMostTraceSmem) {
     static std::mutex m;
-    static std::unordered_map<size_t, int> cache;
-    const size_t key = ((size_t)(void*)kernel) ^ ((size_t)blockSize << 48) ^ (smem << 20);
-    int perSm = 0;
-    {
-        std::lock_guard<std::mutex> g(m);
-        auto it = cache.find(key);
-        if (it != cache.end()) perSm = it->second;
+    static std::map<std::tuple<const void*, int, int, size_t>, int> cache;  // kernel, device, block, shared memory
+    static std::set<std::pair<const void*, int>> optedIn;
+    const void* k = (const void*)kernel;
+    const int device = deviceOf(c);
+    std::lock_guard<std::mutex> g(m);
+    if (smem > 48 * 1024 && !optedIn.count({k, device})) {
+        GRT_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mostSmem));
+        optedIn.insert({k, device});
     }
-    if (perSm == 0) {
-        // above 48 KB (deep stacks in large blocks) a kernel has to opt in: to the most any
-        // call can ask for, so that no later call lowers it
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)std::max<size_t>(smem, 256 * traceSmemWords(false, false, 32, 8) * sizeof(uint32_t)));
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, kernel, blockSize, smem) != cudaSuccess || perSm < 1)
-            perSm = 1;
-        std::lock_guard<std::mutex> g(m);
-        cache[key] = perSm;
-    }
-    return LaunchShape{blockSize, perSm * smCount(c)};
+    int& perSm = cache[{k, device, blockSize, smem}];
+    if (perSm == 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perSm, k, blockSize, smem) != cudaSuccess ||
+                       perSm < 1))
+        perSm = 1;
+    *out = LaunchShape{blockSize, perSm * smCount(c)};
+    return GRT_SUCCESS;
 }
 
 static grtError resolveOptions(const grtTraceOptions* opt, int* blockSize, uint32_t* sh, uint32_t* gl) {
@@ -705,7 +711,9 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
         traceKernelFor<ANY, false>(isScene, walkFormats(P, isScene), n, &kernel);
     cudaStream_t s = (cudaStream_t)stream;
     const size_t smem = (size_t)bs * traceSmemWords(ANY, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
-    LaunchShape L = persistentShape(c, kernel, bs, smem);
+    LaunchShape L;
+    e = persistentShape(c, kernel, bs, smem, &L);
+    if (e != GRT_SUCCESS) return e;
     L.blocks = traceBlocks(c, opt, P, L, n, ANY, isScene);
     e = bindGlobalStack(c, opt, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
@@ -792,7 +800,9 @@ grtError grtTraceClosestNoAlloc(grtContext ctx, grtScene scene, grtGeometry geom
     else
         traceKernelFor<false, false>(isScene, walkFormats(P, isScene), rayCount, &kernel);
     const size_t smem = (size_t)bs * traceSmemWords(false, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
-    LaunchShape L = persistentShape(c, kernel, bs, smem);
+    LaunchShape L;
+    e = persistentShape(c, kernel, bs, smem, &L);
+    if (e != GRT_SUCCESS) return e;
     L.blocks = std::min<int>(L.blocks, (int)ceilDiv(rayCount, bs / 32));
     L.blocks = std::max(1, std::min<int>(L.blocks, (int)(capacity / perBlock)));  // the grid shrinks to fit
     P.counter = reinterpret_cast<unsigned long long*>(base);
@@ -817,7 +827,9 @@ grtError grtGetTraceGlobalStackSize(grtContext ctx, const grtTraceOptions* optio
     // every variant a launch may choose, each with its own shared memory
     auto most = [&](auto k, bool any, bool scene, int w) {
         const size_t sm = (size_t)bs * traceSmemWords(any, scene, sh, w) * sizeof(uint32_t);
-        threads = std::max(threads, persistentShape(c, k, bs, sm).blocks * bs);
+        LaunchShape L{bs, 0};
+        if (e == GRT_SUCCESS) e = persistentShape(c, k, bs, sm, &L);
+        threads = std::max(threads, L.blocks * bs);
     };
     most(traceKernel<false, false, false>, false, false, 4), most(traceKernel<false, true, false>, false, true, 4);
     most(traceKernel<true, false, false>, true, false, 4), most(traceKernel<true, true, false>, true, true, 4);
@@ -838,6 +850,7 @@ grtError grtGetTraceGlobalStackSize(grtContext ctx, const grtTraceOptions* optio
     most(aoTraceKernel<false>, true, true, 4), most(aoTraceKernel<true>, true, true, 4);
     most(aoTraceKernel<false, kFmWide8>, true, true, 8), most(aoTraceKernel<true, kFmWide8>, true, true, 8);
     most(aoTraceKernel<false, kFmQuant>, true, true, 4), most(aoTraceKernel<true, kFmQuant>, true, true, 4);
+    if (e != GRT_SUCCESS) return e;
     *sizeBytes = (size_t)threads * gl * sizeof(uint32_t);
     return GRT_SUCCESS;
 }
@@ -984,7 +997,9 @@ grtError grtTraceAmbientOcclusion(grtContext ctx, grtScene scene, const grtRay* 
                                            : (count ? aoTraceKernel<true> : aoTraceKernel<false>);
     cudaStream_t s = (cudaStream_t)stream;
     const size_t smem = (size_t)bs * traceSmemWords(true, true, P.sharedDepth, slotsOf(walkFormats(P, true))) * sizeof(uint32_t);
-    LaunchShape L = persistentShape(c, kernel, bs, smem);
+    LaunchShape L;
+    e = persistentShape(c, kernel, bs, smem, &L);
+    if (e != GRT_SUCCESS) return e;
     // scratch after the global stack: the hit count (256 B), the list of hit pixels and
     // their AO frames (48 B each)
     void* extra = nullptr;
@@ -1305,9 +1320,11 @@ static grtError launchShadeForward(Context* c, bool scene, TraceParams& P, const
             ? (scene ? shadeForwardKernel<true, kFmQuant> : shadeForwardKernel<false, kFmQuant>)
             : (scene ? shadeForwardKernel<true> : shadeForwardKernel<false>);
     const size_t smem = (size_t)bs * traceSmemWords(true, scene, P.sharedDepth, slotsOf(walkFormats(P, scene))) * sizeof(uint32_t);
-    LaunchShape L = persistentShape(c, kernel, bs, smem);
+    LaunchShape L;
+    grtError e = persistentShape(c, kernel, bs, smem, &L);
+    if (e != GRT_SUCCESS) return e;
     L.blocks = traceBlocks(c, options, P, L, S.n, true, scene);
-    grtError e = bindGlobalStack(c, options, L.blocks * bs, P);
+    e = bindGlobalStack(c, options, L.blocks * bs, P);
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);
     kernel<<<L.blocks, bs, smem, s>>>(P, S);
@@ -1366,8 +1383,9 @@ static grtError shadeBackward(grtContext ctx, grtScene scene, grtGeometry geom, 
         scene ? (priv ? shadeBackwardKernel<true, true> : shadeBackwardKernel<true, false>)
               : (priv ? shadeBackwardKernel<false, true> : shadeBackwardKernel<false, false>);
     const size_t smem = priv ? (size_t)nv * 24 : 0;
-    if (smem > 48 * 1024) GRT_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    LaunchShape L = persistentShape(c, kernel, bs, smem);
+    LaunchShape L;
+    e = persistentShape(c, kernel, bs, smem, &L, kShadePrivateBytes);
+    if (e != GRT_SUCCESS) return e;
     // the adjoint traces nothing: 8 blocks per SM keep each block's share of pixels large
     // next to its pass over the private copy
     L.blocks = std::min(L.blocks, 8 * smCount(c));
