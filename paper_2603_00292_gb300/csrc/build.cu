@@ -827,12 +827,14 @@ static grtError sortCodes(Context* ctx, BvhObject* o, const BuildLayout& L, char
     if (o->mortonBits == 30) {
         uint32_t* const keys[2] = {(uint32_t*)(temp + L.keys[0]), (uint32_t*)(temp + L.keys[1])};
         mortonKernel<uint32_t, 10><<<countBlocks(ctx, n), kCountThreads, 0, s>>>(cen, n, bounds, keys[0], S.hist);
+        GRT_LAUNCH_CHECK();
         err = sortPasses<uint32_t>(ctx, keys, vals, n, L.passes, S, true, s);
     } else {
         unsigned long long* const keys[2] = {(unsigned long long*)(temp + L.keys[0]),
                                              (unsigned long long*)(temp + L.keys[1])};
         mortonKernel<unsigned long long, 21><<<countBlocks(ctx, n), kCountThreads, 0, s>>>(cen, n, bounds, keys[0],
                                                                                          S.hist);
+        GRT_LAUNCH_CHECK();
         err = sortPasses<unsigned long long>(ctx, keys, vals, n, L.passes, S, true, s);
     }
     if (err != GRT_SUCCESS) return err;
@@ -865,17 +867,18 @@ static grtError launchEmitFitT(Context* c, BvhObject* o, const BuildLayout& L, c
     in.tops = (uint4*)(temp + L.tops);
     in.counts = (uint32_t*)(in.tops + (size_t)emitLists(P.n) * kTopMax);
     emitFitKernel<K, KIND><<<lists, kEmitLeaves, 0, s>>>(E, keys, in);
+    GRT_LAUNCH_CHECK();  // a further launch reads the lists and nodes of the one before
     noteLaunches(1);
     while (lists > 1) {
         const TopLists out{in.tops + (size_t)lists * kTopMax, in.counts + lists};
         const uint32_t next = ceilDiv(lists, kTopFan);
         emitTopKernel<K, KIND><<<next, kTopThreads, sizeof(TopShared), s>>>(E, keys, in, lists, out,
                                                                            &workspace(c)->error);
+        GRT_LAUNCH_CHECK();
         noteLaunches(1);
         in = out;
         lists = next;
     }
-    GRT_LAUNCH_CHECK();
     return GRT_SUCCESS;
 }
 

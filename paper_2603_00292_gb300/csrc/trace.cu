@@ -719,8 +719,11 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
     if (e != GRT_SUCCESS) return e;
     P.counter = nextCounter(c);
     kernel<<<L.blocks, bs, smem, s>>>(P);
-    if (!ANY) refineKernel<<<refineBlocks(n), 256, 0, s>>>(P);
-    GRT_LAUNCH_CHECK();
+    GRT_LAUNCH_CHECK();  // a refused walk leaves no records to refine
+    if (!ANY) {
+        refineKernel<<<refineBlocks(n), 256, 0, s>>>(P);
+        GRT_LAUNCH_CHECK();
+    }
     noteLaunches(ANY ? 1 : 2);
     return GRT_SUCCESS;
 }
@@ -810,6 +813,7 @@ grtError grtTraceClosestNoAlloc(grtContext ctx, grtScene scene, grtGeometry geom
     P.globalStride = (uint32_t)(L.blocks * bs);
     cudaStream_t s = (cudaStream_t)stream;
     kernel<<<L.blocks, bs, smem, s>>>(P);
+    GRT_LAUNCH_CHECK();  // a refused walk leaves no records to refine
     refineKernel<<<refineBlocks(rayCount), 256, 0, s>>>(P);
     GRT_LAUNCH_CHECK();
     noteLaunches(2);
@@ -1013,6 +1017,7 @@ grtError grtTraceAmbientOcclusion(grtContext ctx, grtScene scene, const grtRay* 
     P.counter = nextCounter(c);
     GRT_CUDA(cudaMemsetAsync(listCount, 0, sizeof(uint32_t), s));
     aoCompactKernel<<<ceilDiv(pixelCount, 256), 256, 0, s>>>(P, pixelCount, list, listCount, counts, frames);
+    GRT_LAUNCH_CHECK();
     kernel<<<L.blocks, bs, smem, s>>>(P, list, listCount, counts, frames);
     aoFinishKernel<<<smCount(c) * 4, 256, 0, s>>>(list, listCount, samplesPerPixel, ao);
     GRT_LAUNCH_CHECK();
