@@ -176,6 +176,7 @@ struct ChunkRaySource {
     uint32_t base, n;
     __device__ unsigned long long count() const { return n; }
     __device__ uint32_t warps() const { return blockDim.x >> 5; }  // one block takes the chunk
+    __device__ uint32_t warp() const { return threadIdx.x >> 5; }
     __device__ bool begin(uint32_t i, const TraceParams& Q, Stack& st, RayState& s) const {
         const size_t r = (size_t)base + i;
         const float4 a = Q.rays[2 * r], b = Q.rays[2 * r + 1];

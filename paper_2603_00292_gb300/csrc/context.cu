@@ -15,7 +15,7 @@ struct Context {
     int device;
     int sms;
     DeviceWorkspace* dWork;
-    unsigned nextSlot;
+    unsigned nextSlot, nextCaptureSlot;
     void* scratch;        // traversal global-stack spill area (grown on demand)
     size_t scratchBytes;
     void* aux;            // buffers passed between the launches of one call (grown on demand)
@@ -23,10 +23,13 @@ struct Context {
     std::mutex lock;
 };
 
-unsigned long long* nextCounter(Context* c) {
+unsigned long long* nextCounter(Context* c, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s && cudaStreamIsCapturing(s, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
     std::lock_guard<std::mutex> g(c->lock);
-    const unsigned slot = c->nextSlot++ % kCounterSlots;
-    return c->dWork->counters[slot];
+    if (cap != cudaStreamCaptureStatusNone)
+        return c->dWork->counters + kCounterSlots + c->nextCaptureSlot++ % kCaptureSlots;
+    return c->dWork->counters + c->nextSlot++ % kCounterSlots;
 }
 
 grtError contextAux(Context* c, size_t bytes, void** ptr) {

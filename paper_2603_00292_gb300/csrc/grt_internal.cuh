@@ -69,12 +69,14 @@ static_assert(sizeof(InstanceRecord) == 128, "instance record size");
 // Device error word values are grtError codes; the first nonzero one latched wins
 // by atomicCAS from 0.
 constexpr int kCounterSlots = 256;
+constexpr int kCaptureSlots = 1024;
 struct DeviceWorkspace {
     uint32_t error;
     uint32_t pad[31];
     unsigned long long stats[16];  // traversal statistics (grtTraceStatistics order)
-    // per-launch work counters (round robin): items taken, blocks done; zero between launches
-    unsigned long long counters[kCounterSlots][2];
+    // per-launch work counters, round robin: first those of launches issued at once, then those
+    // of captured launches, which keep theirs for every replay
+    unsigned long long counters[kCounterSlots + kCaptureSlots];
 };
 
 // ------------------------------------------------------------------ host helpers
@@ -109,7 +111,8 @@ inline unsigned ceilDiv(size_t a, size_t b) { return (unsigned)((a + b - 1) / b)
 struct Context;
 Context* asContext(grtContext c);
 DeviceWorkspace* workspace(Context* c);
-unsigned long long* nextCounter(Context* c);  // a work counter slot, zero (kernels leave theirs at zero)
+// A work counter slot for a launch on s, to be zeroed on s before it.
+unsigned long long* nextCounter(Context* c, cudaStream_t s);
 // Caller-or-context global stack memory for traversal spills (grown on demand).
 grtError contextScratch(Context* c, size_t bytes, void** ptr);
 // Context memory for buffers one call passes between its own launches (grown on demand;

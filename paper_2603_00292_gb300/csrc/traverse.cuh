@@ -1424,24 +1424,15 @@ __device__ __forceinline__ float3 aoDirection(const AoFrame& F, uint64_t seed, u
 }
 
 // Lanes of a warp that take items: all of them, unless the grid's warps could take every item
-// at once with fewer than kSpreadBelow each. The rays of a warp take turns whenever they are at different steps,
-// so a small launch ends sooner with them spread out (5,184 rays on a 1,280-triangle mesh:
-// 40 -> 31 us a call); from about 8 a warp on, the work itself counts again.
+// at once with fewer than kSpreadBelow each. The rays of a warp take turns whenever they are at
+// different steps, so a small launch ends sooner with them spread out (5,184 rays on a
+// 1,280-triangle mesh: 40 -> 29 us a call); from about 8 a warp on, the work itself counts
+// again. Such a launch needs no work counter: a warp's items follow from its number.
 constexpr uint32_t kSpreadBelow = 8;
-__device__ __forceinline__ uint32_t itemLanes(unsigned long long total, uint32_t warps) {
+__host__ __device__ __forceinline__ uint32_t itemLanes(unsigned long long total, uint32_t warps) {
     if (total >= (unsigned long long)kSpreadBelow * warps) return 0xffffffffu;
     const uint32_t per = ((uint32_t)total + warps - 1u) / warps;
     return (1u << max(per, 1u)) - 1u;
-}
-
-// The end of a launch's work: the last block to come here puts the work counter back to zero
-// for its next use, so that no launch needs a memset before it.
-__device__ __forceinline__ void releaseCounter(unsigned long long* counter) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();  // this block's takes from the counter come before its arrival
-        if (atomicAdd(counter + 1, 1ull) + 1ull == gridDim.x) counter[0] = 0ull, counter[1] = 0ull;
-    }
 }
 
 // Refill loop with one traversal step per lane per iteration (node visits test their
@@ -1464,10 +1455,10 @@ __device__ __forceinline__ void refillLoopPerRay(const TraceParams& P, Stack& st
         while (!exhausted && (uint32_t)__popc(live) <= P.refillBelow) {
             const uint32_t idle = ~live & lanes;
             if (idle == 0) break;
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(P.counter, (unsigned long long)__popc(idle));
+            unsigned long long base = src.warp() * __popc(lanes);  // fewer lanes: each warp takes its items, once
+            if (lanes == 0xffffffffu && lane == 0) base = atomicAdd(P.counter, (unsigned long long)__popc(idle));
             base = __shfl_sync(0xffffffffu, base, 0);
-            if (base + __popc(idle) >= total || ~lanes) exhausted = true;  // fewer lanes: each warp takes once
+            if (base + __popc(idle) >= total || ~lanes) exhausted = true;
             if ((idle >> lane) & 1u) {
                 const unsigned long long mine = base + __popc(idle & ltMask);
                 if (mine < total && src.begin((uint32_t)mine, P, st, s)) {
@@ -1610,7 +1601,7 @@ __device__ __forceinline__ uint32_t nextState(const TraceParams& P, Stack& st, R
 // to P.refillBelow or fewer, idle lanes take fresh items from the global queue with one
 // atomic per warp. Src supplies the items:
 //   count()             number of items (may be read from device memory)
-//   warps()             number of warps that share them
+//   warps(), warp()     number of warps that share them, and this one's among them
 //   begin(i, P, st, s)  set up item i's ray in s; false if the item has no ray
 //   finish(i, s)        consume item i's result s.best
 // Any-hit queries (shadow and ambient-occlusion rays) take the per-ray form instead, which fits
@@ -1640,10 +1631,10 @@ __device__ __forceinline__ void refillLoop(const TraceParams& P, Stack& st, Src&
         while (!exhausted && (uint32_t)__popc(live) <= P.refillBelow) {
             const uint32_t idle = ~live & lanes;
             if (idle == 0) break;
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(P.counter, (unsigned long long)__popc(idle));
+            unsigned long long base = src.warp() * __popc(lanes);  // fewer lanes: each warp takes its items, once
+            if (lanes == 0xffffffffu && lane == 0) base = atomicAdd(P.counter, (unsigned long long)__popc(idle));
             base = __shfl_sync(0xffffffffu, base, 0);
-            if (base + __popc(idle) >= total || ~lanes) exhausted = true;  // fewer lanes: each warp takes once
+            if (base + __popc(idle) >= total || ~lanes) exhausted = true;
             if ((idle >> lane) & 1u) {
                 const unsigned long long mine = base + __popc(idle & ltMask);
                 if (mine < total && src.begin((uint32_t)mine, P, st, s)) {
@@ -1717,6 +1708,7 @@ __device__ __forceinline__ void refillLoop(const TraceParams& P, Stack& st, Src&
 // A source whose items are shared by every warp of the grid.
 struct GridSource {
     __device__ uint32_t warps() const { return gridDim.x * (blockDim.x >> 5); }
+    __device__ uint32_t warp() const { return (blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
 };
 
 // Items = rays of a ray buffer; results = hit records.
