@@ -1250,7 +1250,8 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
 
 // Repeated BUILDs of a geometry from the same buffers replay a CUDA graph of the launch
 // sequence. Every kernel argument is a function of the build input (addresses, strides,
-// counts), the temporary buffer, the object's own arrays and the device, so a graph
+// counts), the temporary buffer, the object's own arrays, the device and the context's
+// error word (the sort's and the emission's waits and checks latch there), so a graph
 // captured once serves every later build with the same description: new vertex data in
 // the same buffers is read by the replay. The graph is captured on a private stream and
 // launched on the caller's; a different description captures again, and a caller's
@@ -1258,6 +1259,7 @@ static grtError issueGeometryBuild(Context* c, BvhObject* o, uint32_t op, const 
 struct BuildKey {
     grtGeometryBuildInput input;
     const void* temp;
+    const uint32_t* error;
     int device;
     uint32_t radius;
     bool operator==(const BuildKey& k) const { return std::memcmp(this, &k, sizeof(*this)) == 0; }
@@ -1297,6 +1299,7 @@ static grtError replayOrCaptureBuild(Context* c, BvhObject* o, const grtGeometry
     else
         key.input.aabbList = input->aabbList;
     key.temp = t;
+    key.error = &workspace(c)->error;
     key.device = deviceOf(c);
     key.radius = radius;
     std::lock_guard<std::mutex> g(g_buildGraphLock);
