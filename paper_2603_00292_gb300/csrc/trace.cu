@@ -614,9 +614,10 @@ static grtError prepareTrace(Context* c, grtScene scene, grtGeometry geom, grtFu
     return GRT_SUCCESS;
 }
 
-// Global stack for `threads` threads (the caller's buffer or the context's scratch),
-// plus optionally `extraBytes` more of context scratch returned in *extra.
-static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int threads, TraceParams& P,
+// Global stack for the `threads` threads of a trace of `items` items (the caller's buffer or
+// the context's scratch), plus optionally `extraBytes` more of context scratch returned in
+// *extra.
+static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int threads, uint32_t items, TraceParams& P,
                                 size_t extraBytes = 0, void** extra = nullptr) {
     const size_t need = alignUp((size_t)threads * P.globalDepth * sizeof(uint32_t), 256);
     P.globalStride = (uint32_t)threads;
@@ -629,9 +630,11 @@ static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int thre
         *extra = p;
         return e;
     }
-    // at the usual depths the area is made for the largest grid at once, so that no later
-    // trace of another kind or size grows it (growing waits for the device)
-    const size_t most = P.globalDepth <= 64 ? (size_t)smCount(c) * 2048 * P.globalDepth * sizeof(uint32_t) : 0;
+    // The area is made for the largest grid of any kind over as many items (a warp for each, up
+    // to 1,024 threads an SM at the fewest registers, 64), so that no later trace of another
+    // kind grows it: growing waits for the device, and fails under capture. 40 MB at the default
+    // depth and 152 SMs, from 4,864 items on.
+    const size_t most = std::min((size_t)smCount(c) * 1024, 32 * (size_t)items) * P.globalDepth * sizeof(uint32_t);
     grtError e = contextScratch(c, std::max<size_t>(std::max(need, most) + extraBytes, 256), &p);
     P.globalStack = (uint32_t*)p;
     if (extraBytes) *extra = static_cast<char*>(p) + need;
@@ -722,7 +725,7 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
     e = persistentShape(c, kernel, bs, smem, &L);
     if (e != GRT_SUCCESS) return e;
     L.blocks = traceBlocks(c, opt, P, L, n, ANY, isScene);
-    e = bindGlobalStack(c, opt, L.blocks * bs, P);
+    e = bindGlobalStack(c, opt, L.blocks * bs, n, P);
     if (e != GRT_SUCCESS) return e;
     e = bindCounter(c, P, n, L, s);
     if (e != GRT_SUCCESS) return e;
@@ -1017,7 +1020,8 @@ grtError grtTraceAmbientOcclusion(grtContext ctx, grtScene scene, const grtRay* 
     // together), the list of hit pixels and their AO frames (48 B each)
     void* extra = nullptr;
     const size_t listBytes = alignUp(4 * (size_t)pixelCount, 256);
-    e = bindGlobalStack(c, options, L.blocks * bs, P, 256 + listBytes + 48 * (size_t)pixelCount, &extra);
+    e = bindGlobalStack(c, options, L.blocks * bs, pixelCount * samplesPerPixel, P,
+                        256 + listBytes + 48 * (size_t)pixelCount, &extra);
     if (e != GRT_SUCCESS) return e;
     uint32_t* listCount = static_cast<uint32_t*>(extra);
     uint32_t* list = reinterpret_cast<uint32_t*>(static_cast<char*>(extra) + 256);
@@ -1338,7 +1342,7 @@ static grtError launchShadeForward(Context* c, bool scene, TraceParams& P, const
     grtError e = persistentShape(c, kernel, bs, smem, &L);
     if (e != GRT_SUCCESS) return e;
     L.blocks = traceBlocks(c, options, P, L, S.n, true, scene);
-    e = bindGlobalStack(c, options, L.blocks * bs, P);
+    e = bindGlobalStack(c, options, L.blocks * bs, S.n, P);
     if (e != GRT_SUCCESS) return e;
     e = bindCounter(c, P, S.n, L, s);
     if (e != GRT_SUCCESS) return e;
