@@ -484,12 +484,21 @@ static grtError launchNodeFormats(const BvhObject* o, cudaStream_t s) {
 // Up to kSmallBuild primitives (kSmallScene instances) a build runs in one block of
 // kSmallBuildThreads threads, as one launch, instead of a graph of some nine grid-wide
 // launches whose cost is their own latency at this size. The threshold is where the measured
-// times cross (us, one block against the graph, 30-bit codes): 512 triangles 35 / 35, 768 43 /
-// 41, 1,024 49 / 43, 1,280 67 / 45, 2,048 80 / 45; the first build of a geometry, which also
-// captures its graph, 69 / 100 at 1,024, 83 / 105 at 1,280 and 99 / 103 at 2,048. A top level of 4,000 instances
-// took 0.61 against 0.15 ms (its FP64 instance setup runs on one SM). Up to kSharedFitMax
-// primitives the block keeps the whole build on chip (bitonicSortShared, fitLeafShared).
+// times of repeated builds cross (us, one block against the graph, 30-bit codes): 512
+// triangles 35 / 35, 768 43 / 41, 1,024 49 / 43, 1,280 67 / 45, 2,048 80 / 45. A top level of
+// 4,000 instances took 0.61 against 0.15 ms (its FP64 instance setup runs on one SM). Up to
+// kSharedFitMax primitives the block keeps the whole build on chip (bitonicSortShared,
+// fitLeafShared).
+//
+// Capturing the graph costs another 47 us, which up to kSmallGraph primitives is more than a
+// build: a geometry built once would pay more than the one block does (us, waited for, one
+// block / graph captured and launched / the launches without a graph: 1,025 triangles 68 / 104
+// / 75, 1,280 81 / 104 / 76, 2,048 94 / 104 / 75). There the first build of a description runs
+// in one block up to kSmallFirst and as plain launches above; the second too, and the graph is
+// captured behind it, while the GPU builds, for the builds to come.
 constexpr uint32_t kSmallBuild = 1024;
+constexpr uint32_t kSmallFirst = 1152;
+constexpr uint32_t kSmallGraph = 2048;
 constexpr uint32_t kSmallScene = 1024;
 #ifndef GRT_SMALL_BUILD_THREADS
 #define GRT_SMALL_BUILD_THREADS 1024
@@ -498,11 +507,11 @@ constexpr int kSmallBuildThreads = GRT_SMALL_BUILD_THREADS;
 constexpr int kSmallSceneThreads = 512;  // its FP64 instance setup needs more than 64 registers
 
 // Dynamic shared memory of a single-block build: the radix routines' histograms, or
-// the on-chip path's sort pairs, boxes and counters for kSmallBuild primitives.
+// the on-chip path's sort pairs, boxes and counters for kSmallFirst primitives.
 template <typename K>
 constexpr size_t smallBuildSmemBytes() {
     return std::max(blockBuildSmemWords(kSmallBuildThreads) * sizeof(uint32_t),
-                    std::max(sharedBuildBytes<K>(kSmallBuild), sharedBuildBytes<K>(kSmallScene)));
+                    std::max(sharedBuildBytes<K>(kSmallFirst), sharedBuildBytes<K>(kSmallScene)));
 }
 
 template <typename K, int BITS>
@@ -1266,31 +1275,66 @@ struct BuildKey {
 };
 struct BuildGraph {
     BuildKey key;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec = nullptr;  // null: a small build whose description was met once
     unsigned long long launches = 0;
 };
 static std::mutex g_buildGraphLock;
 static std::unordered_map<const BvhObject*, BuildGraph> g_buildGraphs;
-unsigned long long launchCountNow();  // context.cu
+unsigned long long threadLaunches();  // context.cu
 
+static void eraseBuildGraph(std::unordered_map<const BvhObject*, BuildGraph>::iterator it) {
+    if (it->second.exec) cudaGraphExecDestroy(it->second.exec);
+    g_buildGraphs.erase(it);
+}
 static void dropBuildGraph(const BvhObject* o) {
     std::lock_guard<std::mutex> g(g_buildGraphLock);
     auto it = g_buildGraphs.find(o);
-    if (it == g_buildGraphs.end()) return;
-    cudaGraphExecDestroy(it->second.exec);
-    g_buildGraphs.erase(it);
+    if (it != g_buildGraphs.end()) eraseBuildGraph(it);
+}
+
+// A build in one block, which initialises its own scratch.
+static grtError issueSmallBuild(Context* c, BvhObject* o, const grtGeometryBuildInput* input, const BuildLayout& L,
+                                char* t, const PrimSource& S, cudaStream_t s) {
+    BlockBuild B = blockBuildOf(c, o, L, t, input->type == GRT_PRIMITIVE_TRIANGLE_MESH ? 0u : 1u);
+    B.src = S;
+    return launchSmallBuild(B, s);
+}
+
+// The graph of a build's launches, counted as launched; null where it cannot be made.
+static cudaGraphExec_t captureBuild(Context* c, BvhObject* o, const grtGeometryBuildInput* input, const BuildLayout& L,
+                                    char* t, const PrimSource& S, uint32_t radius) {
+    cudaStream_t cs = nullptr;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaError_t ce = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    if (ce == cudaSuccess) {
+        ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+        grtError e = ce == cudaSuccess
+                         ? issueGeometryBuild(c, o, GRT_BUILD_OPERATION_BUILD, input, L, t, S, cs, radius)
+                         : GRT_ERROR_CUDA;
+        if (ce == cudaSuccess) ce = cudaStreamEndCapture(cs, &graph);
+        if (e == GRT_SUCCESS && ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        cudaStreamDestroy(cs);
+        if (e == GRT_SUCCESS && ce == cudaSuccess) return exec;
+    }
+    cudaGetLastError();
+    if (exec) cudaGraphExecDestroy(exec);
+    return nullptr;
 }
 
 static grtError replayOrCaptureBuild(Context* c, BvhObject* o, const grtGeometryBuildInput* input,
                                      const BuildLayout& L, char* t, const PrimSource& S, cudaStream_t s,
                                      uint32_t radius) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (s && cudaStreamIsCapturing(s, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
-    if (cap != cudaStreamCaptureStatusNone) {  // the caller is capturing: issue directly
-        grtError e = issueGeometryBuild(c, o, GRT_BUILD_OPERATION_BUILD, input, L, t, S, s, radius);
+    auto issue = [&](bool oneBlock) {
+        const grtError e = oneBlock ? issueSmallBuild(c, o, input, L, t, S, s)
+                                    : issueGeometryBuild(c, o, GRT_BUILD_OPERATION_BUILD, input, L, t, S, s, radius);
         if (e == GRT_SUCCESS) o->built = true;
         return e;
-    }
+    };
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s && cudaStreamIsCapturing(s, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
+    if (cap != cudaStreamCaptureStatusNone) return issue(false);  // the caller is capturing
     BuildKey key;
     std::memset(&key, 0, sizeof(key));
     key.input.type = input->type;  // only the fields the launches read
@@ -1302,41 +1346,39 @@ static grtError replayOrCaptureBuild(Context* c, BvhObject* o, const grtGeometry
     key.error = &workspace(c)->error;
     key.device = deviceOf(c);
     key.radius = radius;
+    const bool small = radius == 0 && !o->split && o->leafCount <= kSmallGraph;
     std::lock_guard<std::mutex> g(g_buildGraphLock);
     auto it = g_buildGraphs.find(o);
     if (it != g_buildGraphs.end() && !(it->second.key == key)) {
-        cudaGraphExecDestroy(it->second.exec);
-        g_buildGraphs.erase(it);
+        eraseBuildGraph(it);
         it = g_buildGraphs.end();
     }
-    if (it == g_buildGraphs.end()) {
-        cudaStream_t cs = nullptr;
-        GRT_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        const unsigned long long before = launchCountNow();
-        cudaGraph_t graph = nullptr;
-        cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        grtError e = ce == cudaSuccess
-                         ? issueGeometryBuild(c, o, GRT_BUILD_OPERATION_BUILD, input, L, t, S, cs, radius)
-                         : GRT_ERROR_CUDA;
-        if (ce == cudaSuccess) ce = cudaStreamEndCapture(cs, &graph);
-        cudaGraphExec_t exec = nullptr;
-        if (e == GRT_SUCCESS && ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        cudaStreamDestroy(cs);
-        if (e != GRT_SUCCESS || ce != cudaSuccess) {  // no graph: the launches go straight to s
-            cudaGetLastError();
-            if (exec) cudaGraphExecDestroy(exec);
-            e = issueGeometryBuild(c, o, GRT_BUILD_OPERATION_BUILD, input, L, t, S, s, radius);
-            if (e == GRT_SUCCESS) o->built = true;
-            return e;
-        }
+    const bool met = it != g_buildGraphs.end();
+    if (met && it->second.exec) {
+        noteLaunches((long long)it->second.launches);
+        GRT_CUDA(cudaGraphLaunch(it->second.exec, s));
+        o->built = true;
+        return GRT_SUCCESS;
+    }
+    if (!met) {
         BuildGraph bg;
         bg.key = key;
-        bg.exec = exec;
-        bg.launches = launchCountNow() - before;  // counted once at capture, for this first replay
         it = g_buildGraphs.emplace(o, bg).first;
-    } else {
-        noteLaunches((unsigned)it->second.launches);
+    }
+    if (small) {
+        const grtError e = issue(o->leafCount <= kSmallFirst);
+        if (e != GRT_SUCCESS || !met) return e;
+    }
+    const unsigned long long before = threadLaunches();
+    it->second.exec = captureBuild(c, o, input, L, t, S, radius);
+    it->second.launches = threadLaunches() - before;
+    if (small) {  // built already
+        noteLaunches(-(long long)it->second.launches);
+        return GRT_SUCCESS;
+    }
+    if (!it->second.exec) {  // no graph: the launches go straight to s
+        g_buildGraphs.erase(it);
+        return issue(false);
     }
     GRT_CUDA(cudaGraphLaunch(it->second.exec, s));
     o->built = true;
@@ -1435,13 +1477,10 @@ grtError grtBuildGeometry(grtContext ctx, uint32_t op, const grtGeometryBuildInp
         S.count = o->leafCount;
         S.refs = (const float4*)(t + splitLayoutOf(o, L, radius).refs);
     }
-    if (op == GRT_BUILD_OPERATION_BUILD && n <= kSmallBuild && radius == 0 && !o->split) {  // initialises its own scratch
-        BlockBuild B = blockBuildOf(c, o, L, t, input->type == GRT_PRIMITIVE_TRIANGLE_MESH ? 0u : 1u);
-        B.src = S;
-        e = launchSmallBuild(B, s);
-        if (e != GRT_SUCCESS) return e;
-        o->built = true;
-        return GRT_SUCCESS;
+    if (op == GRT_BUILD_OPERATION_BUILD && n <= kSmallBuild && radius == 0 && !o->split) {
+        e = issueSmallBuild(c, o, input, L, t, S, s);
+        if (e == GRT_SUCCESS) o->built = true;
+        return e;
     }
     if (op == GRT_BUILD_OPERATION_BUILD) return replayOrCaptureBuild(c, o, input, L, t, S, s, radius);
     e = issueGeometryBuild(c, o, op, input, L, t, S, s);

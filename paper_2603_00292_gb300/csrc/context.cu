@@ -70,8 +70,12 @@ static std::unordered_map<const void*, FuncTableObject*> g_tables;
 static std::atomic<unsigned long long> g_launches{0};
 
 int logLevel() { return g_logLevel; }
-void noteLaunches(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
-unsigned long long launchCountNow() { return g_launches.load(); }
+static thread_local unsigned long long t_launches = 0;  // of the calling thread
+void noteLaunches(long long n) {
+    t_launches += (unsigned long long)n;
+    g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed);
+}
+unsigned long long threadLaunches() { return t_launches; }
 
 void logf(int level, const char* fmt, ...) {
     if (!(g_logLevel & level)) return;
