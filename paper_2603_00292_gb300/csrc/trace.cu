@@ -641,6 +641,12 @@ static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int thre
     return e;
 }
 
+// Blocks that a caller's own stack buffer holds.
+static size_t stackBlocks(const grtTraceOptions* opt, const TraceParams& P, int blockSize) {
+    if (!opt || !opt->globalStack || P.globalDepth == 0) return SIZE_MAX;
+    return (opt->globalStackBytes & ~(size_t)255) / ((size_t)blockSize * P.globalDepth * sizeof(uint32_t));
+}
+
 // Blocks of a trace of n items: a warp takes one at least (itemLanes). A caller's own stack
 // buffer keeps the grid to what it holds, down to a block per blockSize items and at most
 // 640 threads an SM for any hits in one geometry, 512 for the others, below which it is
@@ -648,8 +654,8 @@ static grtError bindGlobalStack(Context* c, const grtTraceOptions* opt, int thre
 static int traceBlocks(Context* c, const grtTraceOptions* opt, const TraceParams& P, LaunchShape L, uint32_t n,
                        bool any, bool scene) {
     const int spread = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize / 32));
-    if (!opt || !opt->globalStack || P.globalDepth == 0) return spread;
-    const size_t fits = (opt->globalStackBytes & ~(size_t)255) / ((size_t)L.blockSize * P.globalDepth * sizeof(uint32_t));
+    const size_t fits = stackBlocks(opt, P, L.blockSize);
+    if (fits == SIZE_MAX) return spread;
     const int sms = smCount(c) * ((any && !scene ? 640 : 512) / L.blockSize);
     const int least = std::min(std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize)), sms);
     return std::max(least, (int)std::min<size_t>(fits, (size_t)spread));
@@ -683,10 +689,14 @@ static int walkFormats(const TraceParams& P, bool scene) {
 // against phased): 2 M camera rays 150 / 186, 1.9 M 388 / 437, 3 M through 1 M spheres 4,510 /
 // 4,570; 733,391 through 41,718 spheres 1,203 / 1,158, 303,000 68 / 61, 86,000 54 / 48.
 constexpr uint32_t kPerRayFrom = 1u << 20;
+// And the threads an SM that its grid must get: with fewer (a bounded stack buffer, blocks of
+// 256) the phased form is faster there too. 2 M rays through 131,072 triangles / 1 M spheres, us
+// per ray against phased: at 431 threads 1,152 / 3,109 against 880 / 2,215 (without allocation),
+// at 768 865 / 2,194 against 788 / 1,950 (blocks of 256, shared depth 32).
+constexpr int kPerRayThreads = 896;
 
 template <bool ANY, bool COUNT>
-static void traceKernelFor(bool scene, int fm, uint32_t n, void (**k)(TraceParams)) {
-    const bool perRay = !ANY && n >= kPerRayFrom;
+static void traceKernelFor(bool scene, int fm, bool perRay, void (**k)(TraceParams)) {
     if (fm == kFmWide8)
         *k = scene ? traceKernel<ANY, true, COUNT, kFmWide8> : traceKernel<ANY, false, COUNT, kFmWide8>;
     else if (fm == kFmQuant)
@@ -697,6 +707,24 @@ static void traceKernelFor(bool scene, int fm, uint32_t n, void (**k)(TraceParam
         *k = scene    ? traceKernel<ANY, true, COUNT>
              : perRay ? traceKernel<ANY, false, COUNT, kFmPlain, ANY>
                       : traceKernel<ANY, false, COUNT>;
+}
+
+// The kernel of a trace of n rays, its shared memory and its persistent grid, of which the
+// stack memory holds no more than `bound` blocks.
+template <bool ANY>
+static grtError chooseTraceKernel(Context* c, const TraceParams& P, bool scene, bool count, uint32_t n, int bs,
+                                  size_t bound, void (**kernel)(TraceParams), size_t* smem, LaunchShape* L) {
+    const int fm = walkFormats(P, scene);
+    *smem = (size_t)bs * traceSmemWords(ANY, scene, P.sharedDepth, slotsOf(fm)) * sizeof(uint32_t);
+    for (bool perRay = !ANY && !scene && fm != kFmWide8 && n >= kPerRayFrom;; perRay = false) {
+        if (count)
+            traceKernelFor<ANY, true>(scene, fm, perRay, kernel);
+        else
+            traceKernelFor<ANY, false>(scene, fm, perRay, kernel);
+        const grtError e = persistentShape(c, *kernel, bs, *smem, L);
+        if (e != GRT_SUCCESS || !perRay) return e;
+        if (std::min((size_t)L->blocks, bound) * bs >= (size_t)kPerRayThreads * smCount(c)) return GRT_SUCCESS;
+    }
 }
 
 template <bool ANY>
@@ -714,15 +742,11 @@ static grtError launchTrace(grtContext ctx, grtScene scene, grtGeometry geom, co
     P.rays = (const float4*)rays;
     P.hits = (uint32_t*)hits;
     P.count = n;
-    void (*kernel)(TraceParams) = nullptr;
-    if (count)
-        traceKernelFor<ANY, true>(isScene, walkFormats(P, isScene), n, &kernel);
-    else
-        traceKernelFor<ANY, false>(isScene, walkFormats(P, isScene), n, &kernel);
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t smem = (size_t)bs * traceSmemWords(ANY, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
+    void (*kernel)(TraceParams) = nullptr;
+    size_t smem = 0;
     LaunchShape L;
-    e = persistentShape(c, kernel, bs, smem, &L);
+    e = chooseTraceKernel<ANY>(c, P, isScene, count, n, bs, stackBlocks(opt, P, bs), &kernel, &smem, &L);
     if (e != GRT_SUCCESS) return e;
     L.blocks = traceBlocks(c, opt, P, L, n, ANY, isScene);
     e = bindGlobalStack(c, opt, L.blocks * bs, n, P);
@@ -809,13 +833,9 @@ grtError grtTraceClosestNoAlloc(grtContext ctx, grtScene scene, grtGeometry geom
     P.hits = (uint32_t*)hits;
     P.count = rayCount;
     void (*kernel)(TraceParams) = nullptr;
-    if (count)
-        traceKernelFor<false, true>(isScene, walkFormats(P, isScene), rayCount, &kernel);
-    else
-        traceKernelFor<false, false>(isScene, walkFormats(P, isScene), rayCount, &kernel);
-    const size_t smem = (size_t)bs * traceSmemWords(false, isScene, P.sharedDepth, slotsOf(walkFormats(P, isScene))) * sizeof(uint32_t);
+    size_t smem = 0;
     LaunchShape L;
-    e = persistentShape(c, kernel, bs, smem, &L);
+    e = chooseTraceKernel<false>(c, P, isScene, count, rayCount, bs, capacity / perBlock, &kernel, &smem, &L);
     if (e != GRT_SUCCESS) return e;
     L.blocks = std::min<int>(L.blocks, (int)ceilDiv(rayCount, bs / 32));
     L.blocks = std::max(1, std::min<int>(L.blocks, (int)(capacity / perBlock)));  // the grid shrinks to fit

@@ -63,6 +63,7 @@ def test_calls_do_not_depend_on_the_counters_they_find(own, n):
     ctx, g = own[:2]
     want, grads = _calls(*own, n)
     assert (want[0][:, 1] != -1).sum() > n // 20
+    assert torch.equal(want[0], want[4]) and torch.equal(want[1], want[5])  # with and without allocation
     for _ in range(2):
         torch.cuda.synchronize()
         _leave_traces(ctx, g.handle)
