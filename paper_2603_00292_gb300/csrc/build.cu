@@ -511,15 +511,16 @@ static grtError launchNodeFormats(const BvhObject* o, cudaStream_t s) {
 // kSharedFitMax primitives the block keeps the whole build on chip (bitonicSortShared,
 // fitLeafShared).
 //
-// Capturing the graph costs another 47 us, which up to kSmallGraph primitives is more than a
-// build: a geometry built once would pay more than the one block does (us, waited for, one
-// block / graph captured and launched / the launches without a graph: 1,025 triangles 68 / 104
-// / 75, 1,280 81 / 104 / 76, 2,048 94 / 104 / 75). There the first build of a description runs
-// in one block up to kSmallFirst and as plain launches above; the second too, and the graph is
-// captured behind it, while the GPU builds, for the builds to come.
+// Capturing the graph costs 50 to 70 us, up to kSmallGraph primitives as much as a build: a
+// geometry built once paid more for it than the one block took (us, first build of a geometry,
+// waited for, one block / graph captured and launched / its launches without a graph: 1,025
+// triangles 70 / 112 / 75, 1,280 84 / 126 / 76, 2,048 98 / 125 / 76). There the first builds of a
+// description run in one block up to kSmallFirst and as plain launches above, some 15 us longer
+// than the graph, which is captured once kDirectBuilds of them have cost what it costs.
 constexpr uint32_t kSmallBuild = 1024;
 constexpr uint32_t kSmallFirst = 1152;
 constexpr uint32_t kSmallGraph = 2048;
+constexpr uint32_t kDirectBuilds = 4;
 constexpr uint32_t kSmallScene = 1024;
 #ifndef GRT_SMALL_BUILD_THREADS
 #define GRT_SMALL_BUILD_THREADS 1024
@@ -1296,8 +1297,9 @@ struct BuildKey {
 };
 struct BuildGraph {
     BuildKey key;
-    cudaGraphExec_t exec = nullptr;  // null: a small build whose description was met once
+    cudaGraphExec_t exec = nullptr;
     unsigned long long launches = 0;
+    uint32_t builds = 0;  // issued without a graph
 };
 static std::mutex g_buildGraphLock;
 static std::unordered_map<const BvhObject*, BuildGraph> g_buildGraphs;
@@ -1374,34 +1376,25 @@ static grtError replayOrCaptureBuild(Context* c, BvhObject* o, const grtGeometry
         eraseBuildGraph(it);
         it = g_buildGraphs.end();
     }
-    const bool met = it != g_buildGraphs.end();
-    if (met && it->second.exec) {
-        noteLaunches((long long)it->second.launches);
-        GRT_CUDA(cudaGraphLaunch(it->second.exec, s));
-        o->built = true;
-        return GRT_SUCCESS;
-    }
-    if (!met) {
+    if (it == g_buildGraphs.end()) {
         BuildGraph bg;
         bg.key = key;
         it = g_buildGraphs.emplace(o, bg).first;
     }
-    if (small) {
-        const grtError e = issue(o->leafCount <= kSmallFirst);
-        if (e != GRT_SUCCESS || !met) return e;
+    BuildGraph& G = it->second;
+    if (!G.exec) {
+        if (small && G.builds < kDirectBuilds) {
+            ++G.builds;
+            return issue(o->leafCount <= kSmallFirst);
+        }
+        const unsigned long long before = threadLaunches();
+        G.exec = captureBuild(c, o, input, L, t, S, radius);
+        if (!G.exec) return issue(false);  // no graph: the launches go straight to s
+        G.launches = threadLaunches() - before;  // counted once at capture, for this first replay
+    } else {
+        noteLaunches((unsigned)G.launches);
     }
-    const unsigned long long before = threadLaunches();
-    it->second.exec = captureBuild(c, o, input, L, t, S, radius);
-    it->second.launches = threadLaunches() - before;
-    if (small) {  // built already
-        noteLaunches(-(long long)it->second.launches);
-        return GRT_SUCCESS;
-    }
-    if (!it->second.exec) {  // no graph: the launches go straight to s
-        g_buildGraphs.erase(it);
-        return issue(false);
-    }
-    GRT_CUDA(cudaGraphLaunch(it->second.exec, s));
+    GRT_CUDA(cudaGraphLaunch(G.exec, s));
     o->built = true;
     return GRT_SUCCESS;
 }

@@ -71,9 +71,9 @@ static std::atomic<unsigned long long> g_launches{0};
 
 int logLevel() { return g_logLevel; }
 static thread_local unsigned long long t_launches = 0;  // of the calling thread
-void noteLaunches(long long n) {
-    t_launches += (unsigned long long)n;
-    g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed);
+void noteLaunches(unsigned n) {
+    t_launches += n;
+    g_launches.fetch_add(n, std::memory_order_relaxed);
 }
 unsigned long long threadLaunches() { return t_launches; }
 

@@ -81,7 +81,7 @@ struct DeviceWorkspace {
 
 // ------------------------------------------------------------------ host helpers
 int logLevel();
-void noteLaunches(long long n);  // adds to the process-wide kernel launch count
+void noteLaunches(unsigned n);  // adds to the process-wide kernel launch count
 void logf(int level, const char* fmt, ...);
 
 #define GRT_CUDA(call)                                                                 \

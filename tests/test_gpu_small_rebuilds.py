@@ -1,6 +1,6 @@
 """Builds around the sizes where one block, plain launches and a captured graph take over from
-each other: the first, second and later builds of a description, and builds that change it,
-equal the oracle bit for bit."""
+each other: the first builds of a description, those that replay its graph, and builds that
+change it, equal the oracle bit for bit."""
 import numpy as np
 import pytest
 import torch
@@ -24,7 +24,7 @@ def _boxes(n, seed):
 @pytest.mark.parametrize("bits", [30, 63])
 @pytest.mark.parametrize("flags", [0, grt.GRT_BUILD_WIDE8_NODES])
 def test_builds_of_one_description(gpu, n, bits, flags):
-    cases = [dict(boxes=_boxes(n, k)) for k in range(4)]
+    cases = [dict(boxes=_boxes(n, k)) for k in range(7)]  # the graph is captured for the fifth
     boxes = device_tensor(cases[0]["boxes"])
     g = Geometry(gpu, boxes=boxes, morton_bits=bits, build_flags=flags)
     for case in cases:  # other boxes in the same buffer
@@ -50,7 +50,7 @@ def test_captured_by_the_caller_between_others(gpu, n):
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
         g.build()
-    for _ in range(3):
+    for _ in range(6):
         boxes.copy_(device_tensor(cases[0]["boxes"]))
         g.build()
         check_bit_exact(g, cases[0], 30)
