@@ -17,26 +17,27 @@ namespace grt {
 // FM: the node formats the walk may meet (traverse.cuh): kFmPlain (4-wide only),
 // kFmQuant (4-wide or quantised, read per level) or kFmWide8 (8-wide on every level).
 //
-// PHASED: of a closest hit, the phased form of refillLoop; without it the per-ray form, for
-// 4-slot nodes of one geometry (kPerRayFrom).
+// DENSE: the form with fewer registers and more warps on an SM, of one geometry's 4-slot nodes:
+// any hits at 64 registers, closest hits in the per-ray form at 72 (plain nodes only). Without it
+// any hits have 96, which every one of their values fits, and closest hits take the phased form.
 //
 // Register caps, measured on 4 M rays through 1 M spheres and 64 terrains (us). One geometry,
 // closest per ray: 72 (3,860; 64: 4,160, 76: 4,195, 80: 4,160, 96: 4,580, none: 5,290); any hit:
-// 64 (2,345; 56: 2,570, 68: 2,470, 96: 2,750). Both spill a few words outside the loop's
-// common path for 7 and 8 blocks of 128 threads on an SM instead of 4 and 5. Scenes hold
-// twice the state (the world ray and the level's) and 8-slot visits twice the distances:
-// closest 128 (64 terrains near 592; 104: 655, 96: 648).
-__host__ __device__ constexpr int traceRegisters(bool any, bool scene, int w, bool phased) {
-    return scene ? 128 : any ? (w == 8 ? 96 : 64) : phased ? 128 : 72;
+// 64 (2,345; 56: 2,570, 68: 2,470, 96: 2,750). Both spill (136 and 80 bytes a thread): a shorter
+// launch, whose time is its longest rays', takes the other form (kDenseAnyFrom, kPerRayFrom).
+// Scenes hold twice the state (the world ray and the level's) and 8-slot visits twice the
+// distances: closest 128 (64 terrains near 592; 104: 655, 96: 648).
+__host__ __device__ constexpr int traceRegisters(bool any, bool scene, bool dense) {
+    return scene ? 128 : any ? (dense ? 64 : 96) : dense ? 72 : 128;
 }
 
-template <bool ANY, bool SCENE, bool COUNT, int FM = kFmPlain, bool PHASED = true>
-__global__ void __maxnreg__(traceRegisters(ANY, SCENE, slotsOf(FM), PHASED)) traceKernel(TraceParams P) {
+template <bool ANY, bool SCENE, bool COUNT, int FM = kFmPlain, bool DENSE = false>
+__global__ void __maxnreg__(traceRegisters(ANY, SCENE, DENSE)) traceKernel(TraceParams P) {
     extern __shared__ uint32_t sstack[];
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     Stack st{sstack + threadIdx.x, P.globalStack + gtid, P.sharedDepth, P.globalDepth, P.globalStride, 0};
     RayBufferSource<ANY, SCENE> src{P.count, &P};
-    refillLoop<ANY, SCENE, COUNT, FM, PHASED>(P, st, src);
+    refillLoop<ANY, SCENE, COUNT, FM, !DENSE>(P, st, src);
 }
 
 // The closest hits' t, u, v recomputed in double-float, one thread per ray after traversal so
@@ -278,7 +279,7 @@ struct ShadowSource : GridSource {
             const ShadeHit H = setup(i);
             if (H.nl > 0.0f) {
                 const float3 l = make_float3(S->light[0], S->light[1], S->light[2]);
-                beginRay<SCENE, true>(P, st, s, (H.o + H.d * H.t) + H.nf * 1e-4f, l, 0.0f, INFINITY);
+                beginRay<SCENE, fusedSlab(true, SCENE)>(P, st, s, (H.o + H.d * H.t) + H.nf * 1e-4f, l, 0.0f, INFINITY);
                 return true;
             }
         }
@@ -298,9 +299,9 @@ struct ShadowSource : GridSource {
     }
 };
 
-// One geometry at 72 registers: a 1080p step 426 us, 439 at 80, 440 at 96, 454 at 64.
-template <bool SCENE, int FM = kFmPlain>
-__global__ void __maxnreg__(SCENE ? 128 : 72) shadeForwardKernel(TraceParams P, ShadeParams S) {
+// One geometry's DENSE form at 72 registers: a 1080p step 426 us, 439 at 80, 440 at 96, 454 at 64.
+template <bool SCENE, int FM = kFmPlain, bool DENSE = false>
+__global__ void __maxnreg__(SCENE ? 128 : DENSE ? 72 : 96) shadeForwardKernel(TraceParams P, ShadeParams S) {
     extern __shared__ uint32_t sstack[];
     const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x;
     Stack st{sstack + threadIdx.x, P.globalStack + gtid, P.sharedDepth, P.globalDepth, P.globalStride, 0};
@@ -647,18 +648,25 @@ static size_t stackBlocks(const grtTraceOptions* opt, const TraceParams& P, int 
     return (opt->globalStackBytes & ~(size_t)255) / ((size_t)blockSize * P.globalDepth * sizeof(uint32_t));
 }
 
-// Blocks of a trace of n items: a warp takes one at least (itemLanes). A caller's own stack
-// buffer keeps the grid to what it holds, down to a block per blockSize items and at most
-// 640 threads an SM for any hits in one geometry, 512 for the others, below which it is
-// refused.
+// Blocks that n items fill: with fewer lanes than a warp has, as many warps as there are items
+// (itemLanes); else full warps, so that they spread evenly over the SMs (60,000 any hits on an
+// icosphere's mesh 54 -> 47 us, shading them 72 -> 61).
+static int itemBlocks(const LaunchShape& L, uint32_t n) {
+    const uint32_t warps = (uint32_t)(L.blockSize / 32);
+    return std::min<int>(L.blocks, (int)ceilDiv(n, ~itemLanes(n, L.blocks * warps) ? warps : L.blockSize));
+}
+
+// Blocks of a trace of n items. A caller's own stack buffer keeps the grid to what it holds,
+// down to a block per blockSize items and at most 640 threads an SM for any hits in one
+// geometry, 512 for the others, below which it is refused.
 static int traceBlocks(Context* c, const grtTraceOptions* opt, const TraceParams& P, LaunchShape L, uint32_t n,
                        bool any, bool scene) {
-    const int spread = std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize / 32));
+    const int wanted = itemBlocks(L, n);
     const size_t fits = stackBlocks(opt, P, L.blockSize);
-    if (fits == SIZE_MAX) return spread;
+    if (fits == SIZE_MAX) return wanted;
     const int sms = smCount(c) * ((any && !scene ? 640 : 512) / L.blockSize);
     const int least = std::min(std::min<int>(L.blocks, (int)ceilDiv(n, L.blockSize)), sms);
-    return std::max(least, (int)std::min<size_t>(fits, (size_t)spread));
+    return std::max(least, (int)std::min<size_t>(fits, (size_t)wanted));
 }
 
 // The work counter of a walk of n items on s, cleared there: what an earlier launch left in the
@@ -683,30 +691,41 @@ static int walkFormats(const TraceParams& P, bool scene) {
     return kFmPlain;
 }
 
-// Rays from which closest hits in one geometry (4-slot nodes) take the per-ray form with its
+// Rays from which closest hits in one geometry (plain nodes) take the per-ray form with its
 // 28 warps an SM instead of the phased one with 16. It has more work in flight; the phased
 // form has the shorter chain per ray, which is what a smaller launch waits for (us, per ray
 // against phased): 2 M camera rays 150 / 186, 1.9 M 388 / 437, 3 M through 1 M spheres 4,510 /
-// 4,570; 733,391 through 41,718 spheres 1,203 / 1,158, 303,000 68 / 61, 86,000 54 / 48.
+// 4,570; 733,391 through 41,718 spheres 1,203 / 1,158, 303,000 68 / 61, 86,000 54 / 48. Over
+// quantised nodes the phased form stays faster (2 M uniform rays, an icosphere 1,036 against
+// 1,138, a terrain 760 against 829).
 constexpr uint32_t kPerRayFrom = 1u << 20;
-// And the threads an SM that its grid must get: with fewer (a bounded stack buffer, blocks of
-// 256) the phased form is faster there too. 2 M rays through 131,072 triangles / 1 M spheres, us
+// Items from which any hits and shadow rays in one geometry take the form with more warps and
+// spills (us, 96 registers against 64, 72 shading; uniform rays, icosphere): any 160,000 72 / 66,
+// 250,000 95 / 90, 700,000 224 / 195, but a terrain 80 / 85, 107 / 104, 212 / 190; shading
+// 160,000 86 / 86, 250,000 122 / 112, 700,000 284 / 248, a terrain 51 / 55, 58 / 63, 133 / 118.
+constexpr uint32_t kDenseAnyFrom = 1u << 18;
+// And the threads an SM that their grids must get: with fewer (a bounded stack buffer, blocks of
+// 256) the other form is faster there too. 2 M rays through 131,072 triangles / 1 M spheres, us
 // per ray against phased: at 431 threads 1,152 / 3,109 against 880 / 2,215 (without allocation),
 // at 768 865 / 2,194 against 788 / 1,950 (blocks of 256, shared depth 32).
-constexpr int kPerRayThreads = 896;
+constexpr int kPerRayThreads = 896, kDenseAnyThreads = 1024, kDenseShadeThreads = 896;
+
+static bool fullGrid(Context* c, const LaunchShape& L, size_t bound, int threads) {
+    return std::min((size_t)L.blocks, bound) * L.blockSize >= (size_t)threads * smCount(c);
+}
 
 template <bool ANY, bool COUNT>
-static void traceKernelFor(bool scene, int fm, bool perRay, void (**k)(TraceParams)) {
+static void traceKernelFor(bool scene, int fm, bool dense, void (**k)(TraceParams)) {
     if (fm == kFmWide8)
         *k = scene ? traceKernel<ANY, true, COUNT, kFmWide8> : traceKernel<ANY, false, COUNT, kFmWide8>;
     else if (fm == kFmQuant)
-        *k = scene    ? traceKernel<ANY, true, COUNT, kFmQuant>
-             : perRay ? traceKernel<ANY, false, COUNT, kFmQuant, ANY>
-                      : traceKernel<ANY, false, COUNT, kFmQuant>;
+        *k = scene   ? traceKernel<ANY, true, COUNT, kFmQuant>
+             : dense ? traceKernel<ANY, false, COUNT, kFmQuant, ANY>
+                     : traceKernel<ANY, false, COUNT, kFmQuant>;
     else
-        *k = scene    ? traceKernel<ANY, true, COUNT>
-             : perRay ? traceKernel<ANY, false, COUNT, kFmPlain, ANY>
-                      : traceKernel<ANY, false, COUNT>;
+        *k = scene   ? traceKernel<ANY, true, COUNT>
+             : dense ? traceKernel<ANY, false, COUNT, kFmPlain, true>
+                     : traceKernel<ANY, false, COUNT>;
 }
 
 // The kernel of a trace of n rays, its shared memory and its persistent grid, of which the
@@ -716,14 +735,14 @@ static grtError chooseTraceKernel(Context* c, const TraceParams& P, bool scene, 
                                   size_t bound, void (**kernel)(TraceParams), size_t* smem, LaunchShape* L) {
     const int fm = walkFormats(P, scene);
     *smem = (size_t)bs * traceSmemWords(ANY, scene, P.sharedDepth, slotsOf(fm)) * sizeof(uint32_t);
-    for (bool perRay = !ANY && !scene && fm != kFmWide8 && n >= kPerRayFrom;; perRay = false) {
+    bool dense = !scene && (ANY ? fm != kFmWide8 && n >= kDenseAnyFrom : fm == kFmPlain && n >= kPerRayFrom);
+    for (;; dense = false) {
         if (count)
-            traceKernelFor<ANY, true>(scene, fm, perRay, kernel);
+            traceKernelFor<ANY, true>(scene, fm, dense, kernel);
         else
-            traceKernelFor<ANY, false>(scene, fm, perRay, kernel);
+            traceKernelFor<ANY, false>(scene, fm, dense, kernel);
         const grtError e = persistentShape(c, *kernel, bs, *smem, L);
-        if (e != GRT_SUCCESS || !perRay) return e;
-        if (std::min((size_t)L->blocks, bound) * bs >= (size_t)kPerRayThreads * smCount(c)) return GRT_SUCCESS;
+        if (e != GRT_SUCCESS || !dense || fullGrid(c, *L, bound, ANY ? kDenseAnyThreads : kPerRayThreads)) return e;
     }
 }
 
@@ -837,7 +856,7 @@ grtError grtTraceClosestNoAlloc(grtContext ctx, grtScene scene, grtGeometry geom
     LaunchShape L;
     e = chooseTraceKernel<false>(c, P, isScene, count, rayCount, bs, capacity / perBlock, &kernel, &smem, &L);
     if (e != GRT_SUCCESS) return e;
-    L.blocks = std::min<int>(L.blocks, (int)ceilDiv(rayCount, bs / 32));
+    L.blocks = itemBlocks(L, rayCount);
     L.blocks = std::max(1, std::min<int>(L.blocks, (int)(capacity / perBlock)));  // the grid shrinks to fit
     P.counter = reinterpret_cast<unsigned long long*>(base);
     P.globalStack = reinterpret_cast<uint32_t*>(static_cast<char*>(base) + kNoAllocStackOffset);
@@ -879,10 +898,12 @@ grtError grtGetTraceGlobalStackSize(grtContext ctx, const grtTraceOptions* optio
     most(traceKernel<true, false, false, kFmQuant>, true, false, 4), most(traceKernel<true, true, false, kFmQuant>, true, true, 4);
     most(traceKernel<false, false, true, kFmQuant>, false, false, 4), most(traceKernel<false, true, true, kFmQuant>, false, true, 4);
     most(traceKernel<true, false, true, kFmQuant>, true, false, 4), most(traceKernel<true, true, true, kFmQuant>, true, true, 4);
-    most(traceKernel<false, false, false, kFmPlain, false>, false, false, 4);
-    most(traceKernel<false, false, true, kFmPlain, false>, false, false, 4);
-    most(traceKernel<false, false, false, kFmQuant, false>, false, false, 4);
-    most(traceKernel<false, false, true, kFmQuant, false>, false, false, 4);
+    most(traceKernel<false, false, false, kFmPlain, true>, false, false, 4);
+    most(traceKernel<false, false, true, kFmPlain, true>, false, false, 4);
+    most(traceKernel<true, false, false, kFmPlain, true>, true, false, 4);
+    most(traceKernel<true, false, true, kFmPlain, true>, true, false, 4);
+    most(traceKernel<true, false, false, kFmQuant, true>, true, false, 4);
+    most(traceKernel<true, false, true, kFmQuant, true>, true, false, 4);
     most(aoTraceKernel<false>, true, true, 4), most(aoTraceKernel<true>, true, true, 4);
     most(aoTraceKernel<false, kFmWide8>, true, true, 8), most(aoTraceKernel<true, kFmWide8>, true, true, 8);
     most(aoTraceKernel<false, kFmQuant>, true, true, 4), most(aoTraceKernel<true, kFmQuant>, true, true, 4);
@@ -1351,18 +1372,26 @@ static grtError prepareShade(grtContext ctx, grtScene scene, grtGeometry geom, c
 // The forward shading launch (image and / or visibility from stored hits).
 static grtError launchShadeForward(Context* c, bool scene, TraceParams& P, const ShadeParams& S, int bs,
                                    const grtTraceOptions* options, cudaStream_t s) {
-    void (*kernel)(TraceParams, ShadeParams) =
-        walkFormats(P, scene) == kFmWide8
-            ? (scene ? shadeForwardKernel<true, kFmWide8> : shadeForwardKernel<false, kFmWide8>)
-        : walkFormats(P, scene) == kFmQuant
-            ? (scene ? shadeForwardKernel<true, kFmQuant> : shadeForwardKernel<false, kFmQuant>)
-            : (scene ? shadeForwardKernel<true> : shadeForwardKernel<false>);
-    const size_t smem = (size_t)bs * traceSmemWords(true, scene, P.sharedDepth, slotsOf(walkFormats(P, scene))) * sizeof(uint32_t);
+    const int fm = walkFormats(P, scene);
+    const size_t smem = (size_t)bs * traceSmemWords(true, scene, P.sharedDepth, slotsOf(fm)) * sizeof(uint32_t);
+    void (*kernel)(TraceParams, ShadeParams) = nullptr;
     LaunchShape L;
-    grtError e = persistentShape(c, kernel, bs, smem, &L);
-    if (e != GRT_SUCCESS) return e;
+    for (bool dense = !scene && S.n >= kDenseAnyFrom;; dense = false) {
+        kernel = fm == kFmWide8  ? (scene   ? shadeForwardKernel<true, kFmWide8>
+                                    : dense ? shadeForwardKernel<false, kFmWide8, true>
+                                            : shadeForwardKernel<false, kFmWide8>)
+                 : fm == kFmQuant ? (scene   ? shadeForwardKernel<true, kFmQuant>
+                                     : dense ? shadeForwardKernel<false, kFmQuant, true>
+                                             : shadeForwardKernel<false, kFmQuant>)
+                                  : (scene   ? shadeForwardKernel<true>
+                                     : dense ? shadeForwardKernel<false, kFmPlain, true>
+                                             : shadeForwardKernel<false>);
+        const grtError e = persistentShape(c, kernel, bs, smem, &L);
+        if (e != GRT_SUCCESS) return e;
+        if (!dense || fullGrid(c, L, stackBlocks(options, P, bs), kDenseShadeThreads)) break;
+    }
     L.blocks = traceBlocks(c, options, P, L, S.n, true, scene);
-    e = bindGlobalStack(c, options, L.blocks * bs, S.n, P);
+    grtError e = bindGlobalStack(c, options, L.blocks * bs, S.n, P);
     if (e != GRT_SUCCESS) return e;
     e = bindCounter(c, P, S.n, L, s);
     if (e != GRT_SUCCESS) return e;
