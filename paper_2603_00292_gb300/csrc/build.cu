@@ -1,13 +1,13 @@
-// LBVH construction on the GPU: primitive boxes and centroid bounds, Morton codes,
-// a stable LSD radix sort, Karras hierarchy emission and a bottom-up fit with
-// atomic visit counters, plus the top-level (instance) build.
+// LBVH construction on the GPU: primitive boxes and centroid bounds, Morton codes, a stable
+// LSD radix sort, hierarchy emission and bottom-up fit in blocks of leaves (emit_fit.cuh),
+// plus the top-level (instance) build. Refits and the fit after a clustering build walk up
+// from the leaves with atomic visit counters (fitKernel).
 //
 // Method: the paper describes BVH construction, its surface-area cost and refitting
 // from child boxes (Sec. 6.2) and the geometry / scene build API (Sec. 7.2-7.3). The
-// linear build follows Karras, "Maximizing Parallelism in the Construction of BVHs,
-// Octrees, and k-d Trees" (HPG 2012): node i of the n-1 internal nodes finds its
-// range and split from the sorted codes alone, and leaves walk up to the root,
-// the second child to arrive at a node computing its box.
+// linear build makes the tree and node numbering of Karras, "Maximizing Parallelism in the
+// Construction of BVHs, Octrees, and k-d Trees" (HPG 2012). Builds of one block search each
+// node's range and split in the sorted codes; larger ones find them from the leaves upwards.
 #include <algorithm>
 #include <atomic>
 #include <cstring>

@@ -1,4 +1,5 @@
-// Hierarchy emission and bottom-up fit of a linear BVH in one launch, over the sorted codes.
+// Hierarchy emission and bottom-up fit of a linear BVH in one pass over the sorted codes, of a
+// launch over blocks of leaves and a few that join what remains.
 //
 // The tree and its numbering are Karras's (HPG 2012), found from the leaves upwards
 // (Apetrei, "Fast and Simple Agglomerative LBVH Construction", CGVC 2014). With delta(i) the

@@ -23,8 +23,9 @@ namespace grt {
 //
 // Register caps, measured on 4 M rays through 1 M spheres and 64 terrains (us). One geometry,
 // closest per ray: 72 (3,860; 64: 4,160, 76: 4,195, 80: 4,160, 96: 4,580, none: 5,290); any hit:
-// 64 (2,345; 56: 2,570, 68: 2,470, 96: 2,750). Both spill (136 and 80 bytes a thread): a shorter
-// launch, whose time is its longest rays', takes the other form (kDenseAnyFrom, kPerRayFrom).
+// 64 (2,345; 56: 2,570, 68: 2,470, 96: 2,750). Both keep part of the state on a stack frame of
+// 64 to 136 bytes a thread: a shorter launch, whose time is its longest rays', takes the other
+// form (kDenseAnyFrom, kPerRayFrom).
 // Scenes hold twice the state (the world ray and the level's) and 8-slot visits twice the
 // distances: closest 128 (64 terrains near 592; 104: 655, 96: 648).
 __host__ __device__ constexpr int traceRegisters(bool any, bool scene, bool dense) {

@@ -41,12 +41,11 @@ __host__ __device__ constexpr int slotsOf(int fm) { return (fm & 2) ? 8 : 4; }
 __host__ __device__ constexpr uint32_t pendingCap(int w) { return w == 8 ? 12u : 8u; }
 // Whether a walk's stack keeps each entry's distance, to drop entries behind a hit found since
 // (pushNearest). Closest hits in one geometry: 1 M spheres visit 23.6 nodes a ray for 27.7
-// and, with the rest of its per-ray form,
-// the walk takes 3.77 ms for 4.74. In a scene a ray's stack is short and the entries
-// dropped are few (16.4 nodes for 17.2 on 64 terrains seen from near), for more work at
-// each pop: 609 us against 585.
-// Not for 8-wide nodes: their 19-comparator network and eight keys cost more than the cases
-// they replace (spheres 0.70 to 0.84 of the speed).
+// and, with the rest of its per-ray form, the walk takes 3.77 ms for 4.74. In a scene a
+// ray's stack is short and the entries dropped are few (16.4 nodes for 17.2 on 64 terrains
+// seen from near), for more work at each pop: 609 us against 585.
+// Not for 8-wide nodes: a network of 19 comparators over eight keys cost more than the cases
+// it replaced (spheres 0.70 to 0.84 of the speed).
 __host__ __device__ constexpr bool keepsDistances(bool any, bool scene, int w) { return !any && !scene && w == 4; }
 // Shared memory per thread of a kernel that runs refillLoop, in words: its stack slice of
 // `depth` entries, their distances, and for closest hits the queue of pending leaves.
@@ -1069,37 +1068,28 @@ __device__ __forceinline__ void orderSlots(const TraceParams& P, Stack& st, RayS
         orderChildren(P, st, s, m, tn, c);
 }
 
-// The inner children of a visit of a walk whose stack keeps each entry's distance: the nearest becomes s.next, the others are pushed farthest first. All lanes of a
+// The inner children of a visit of a walk whose stack keeps each entry's distance (4-slot
+// nodes): the nearest becomes s.next, the others are pushed farthest first. All lanes of a
 // warp take the same path whatever their number of hits: keys of the entry distance (as an
-// integer) with the slot in the low bits, none = no hit, a sorting network (Batcher's, 5 or
-// 19 comparators), then predicated stores; a key's child word is read again from the node
+// integer) with the slot in the two low bits, none = no hit, Batcher's sorting network of 5
+// comparators, then predicated stores; a key's child word is read again from the node
 // (an L1 hit) instead of selected among registers. The form with a case for one, two and
 // more hits ran them one after another in nearly every warp (1 M spheres, phased: 4.40 ms
 // against 4.00).
-template <int W>
-__device__ __forceinline__ void pushNearest(const TraceParams& P, Stack& st, RayState& s, int* k, const uint32_t* words) {
-    constexpr int kLow = W - 1, kNoKey = 0x7FFFFFFF;
+__device__ __forceinline__ void pushNearest(const TraceParams& P, Stack& st, RayState& s, int k[4], const uint32_t* words) {
+    constexpr int kLow = 3, kNoKey = 0x7FFFFFFF;
     auto sort = [&](int a, int b) {
         const int x = min(k[a], k[b]);
         k[b] = max(k[a], k[b]);
         k[a] = x;
     };
-    if constexpr (W == 4) {
-        sort(0, 1), sort(2, 3), sort(0, 2), sort(1, 3), sort(1, 2);
-    } else {
-        sort(0, 1), sort(2, 3), sort(4, 5), sort(6, 7);
-        sort(0, 2), sort(1, 3), sort(4, 6), sort(5, 7);
-        sort(1, 2), sort(5, 6);
-        sort(0, 4), sort(1, 5), sort(2, 6), sort(3, 7);
-        sort(2, 4), sort(3, 5);
-        sort(1, 2), sort(3, 4), sort(5, 6);
-    }
+    sort(0, 1), sort(2, 3), sort(0, 2), sort(1, 3), sort(1, 2);
     s.next = k[0] != kNoKey ? __ldg(words + (k[0] & kLow)) : kNone;
     if (k[1] == kNoKey) return;
-    if (st.sp + (W - 1) <= st.shDepth) {
+    if (st.sp + 3 <= st.shDepth) {
         uint32_t* at = st.sh + st.sp * blockDim.x;
 #pragma unroll
-        for (int j = W - 1; j >= 1; --j)
+        for (int j = 3; j >= 1; --j)
             if (k[j] != kNoKey) {
                 at[0] = __ldg(words + (k[j] & kLow));
                 at[st.shDepth * blockDim.x] = (uint32_t)(k[j] & ~kLow);
@@ -1108,7 +1098,7 @@ __device__ __forceinline__ void pushNearest(const TraceParams& P, Stack& st, Ray
             }
     } else {
         bool ok = true;
-        for (int j = W - 1; j >= 1; --j)
+        for (int j = 3; j >= 1; --j)
             if (k[j] != kNoKey) ok &= st.pushAt(__ldg(words + (k[j] & kLow)), __int_as_float(k[j] & ~kLow));
         if (!ok) latchError(P.error, GRT_ERROR_STACK_OVERFLOW);
     }
@@ -1199,7 +1189,7 @@ __device__ __forceinline__ bool stepRay(const TraceParams& P, Stack& st, RayStat
             lm |= h[j] && leaf ? 1u << j : 0u;
             key[j] = h[j] && !leaf ? ((__float_as_int(tn[j]) & ~(W - 1)) | j) : 0x7FFFFFFF;
         }
-        pushNearest<W>(P, st, s, key, words);
+        pushNearest(P, st, s, key, words);
         while (lm) {
             const uint32_t j = (uint32_t)__ffs(lm) - 1u;
             lm &= lm - 1u;
@@ -1437,11 +1427,11 @@ __host__ __device__ __forceinline__ uint32_t itemLanes(unsigned long long total,
     return (1u << max(per, 1u)) - 1u;
 }
 
-// Refill loop with one traversal step per lane per iteration (node visits test their
-// leaves at once): any-hit queries, which stop at their first hit and so gain nothing from
-// queueing leaves, and large launches of closest hits in one geometry. A walk is a chain of loads and dependent
-// arithmetic, 2,000 to 4,500 cycles an iteration, so what counts is how many warps an SM
-// holds: this form needs few registers (see traceKernel's caps).
+// Refill loop with one traversal step per lane per iteration (node visits test their leaves
+// at once): any-hit queries, which stop at their first hit and so gain nothing from queueing
+// leaves, and large launches of closest hits in one geometry. A walk is a chain of loads and
+// dependent arithmetic, 2,000 to 4,500 cycles an iteration, so what counts is how many warps
+// an SM holds: this form needs few registers (see traceKernel's caps).
 template <bool ANY, bool SCENE, bool COUNT, int FM = kFmMixed, class Src>
 __device__ __forceinline__ void refillLoopPerRay(const TraceParams& P, Stack& st, Src& src) {
     const uint32_t lane = threadIdx.x & 31;
@@ -1550,7 +1540,7 @@ __device__ __forceinline__ void visitNode(const TraceParams& P, Stack& st, RaySt
         for (int j = 0; j < W; ++j)
             if (h[j] && (int)c[j] < 0) q.add(c[j] & ~kLeafBit);
     }
-    pushNearest<W>(P, st, s, key, words);
+    pushNearest(P, st, s, key, words);
 }
 
 // The lane's next action after its last one: pops the stack (leaving an instance
@@ -1607,11 +1597,11 @@ __device__ __forceinline__ uint32_t nextState(const TraceParams& P, Stack& st, R
 //   begin(i, P, st, s)  set up item i's ray in s; false if the item has no ray
 //   finish(i, s)        consume item i's result s.best
 // Any-hit queries (shadow and ambient-occlusion rays) take the per-ray form instead, which fits
-// 64 registers, and so do large launches of closest hits in one geometry (without PHASED;
-// 72 registers, see kPerRayFrom in trace.cu). The phased form stays for the smaller ones,
-// for 8-slot nodes, for scenes, where one code path per iteration is worth more (64
-// terrains: far 313 against 351 us, near 565 against 623), and in the batched launch, whose
-// registers its build phases set anyway (24 soups 21.8 against 23.3 ms).
+// 64 registers, and so do large launches of closest hits in one geometry's plain nodes
+// (without PHASED; 72 registers, see kPerRayFrom in trace.cu). The phased form stays for the
+// smaller ones, for quantised and 8-slot nodes, for scenes, where one code path per iteration
+// is worth more (64 terrains: far 313 against 351 us, near 565 against 623), and in the
+// batched launch, whose registers its build phases set anyway (24 soups 21.8 against 23.3 ms).
 template <bool ANY, bool SCENE, bool COUNT, int FM = kFmMixed, bool PHASED = true, class Src>
 __device__ __forceinline__ void refillLoop(const TraceParams& P, Stack& st, Src& src) {
     if constexpr (ANY || (!SCENE && !PHASED && slotsOf(FM) == 4)) {
