@@ -167,64 +167,63 @@ constexpr bool kFusedAllHits = false;
 // Reciprocal direction for the slab tests; a bounds the origins of the level per axis.
 // Fused, neither a reciprocal nor its product with the origin may be infinite: fma(p, inf,
 // -o inf) is a NaN at best, and with an infinite product alone every plane lies on one side.
-// Reciprocals are therefore kept within the power of two that keeps the product below 2^126;
-// the planes of a smaller component then still lie past every t the ray can have, on the
-// right side. The ray's reach bounds that t: for directions shorter than 2^-38, whose rays
-// reach too far, larger reciprocals become infinite instead, and such an axis culls little or
-// nothing. (Without a branch: a test for infinities and a fix-up cost one instruction in eight
-// of a scene's closest hits.)
-constexpr float kSlabReach = 2.74877907e11f;  // 2^38
+// Reciprocals are therefore kept within slabCap, the power of two that keeps the product
+// below 2^126: the planes of a smaller component then lie nearer than they do, on the right
+// side. (Without a branch: a test for infinities and a fix-up cost one instruction in eight of
+// a scene's closest hits.)
 __device__ __forceinline__ float slabCap(float a) {
     return __uint_as_float(0xBD800000u - (__float_as_uint(fmaxf(a, 1.f)) & 0x7F800000u));  // 2^(125 - exponent of a)
 }
-__device__ __forceinline__ float slabClamp(float r, float cap, bool reaches) {
-    return fabsf(r) > cap ? copysignf(reaches ? cap : INFINITY, r) : r;
+__device__ __forceinline__ float slabClamp(float r, float a) {
+    const float cap = slabCap(a);
+    return fabsf(r) > cap ? copysignf(cap, r) : r;
 }
 template <bool FUSED>
 __device__ __forceinline__ float3 slabReciprocal(float3 d, float3 a) {
-    float3 r = make_float3(__frcp_rn(d.x), __frcp_rn(d.y), __frcp_rn(d.z));
-    if constexpr (FUSED) {
-        const bool reaches = fminf(fminf(fabsf(r.x), fabsf(r.y)), fabsf(r.z)) < kSlabReach;
-        r.x = slabClamp(r.x, slabCap(a.x), reaches);
-        r.y = slabClamp(r.y, slabCap(a.y), reaches);
-        r.z = slabClamp(r.z, slabCap(a.z), reaches);
-    }
-    return r;
+    const float3 r = make_float3(__frcp_rn(d.x), __frcp_rn(d.y), __frcp_rn(d.z));
+    return FUSED ? make_float3(slabClamp(r.x, a.x), slabClamp(r.y, a.y), slabClamp(r.z, a.z)) : r;
 }
 
-// A clamped reciprocal is finite, so a ray that lies in a plane of the box itself gets distance
-// 0 for it where the difference form's 0 inf drops it. Planes within `width` of the origin are
-// therefore moved to either side by width |id|. At the largest reciprocal, 2^125, that is 2^63
-// times the least reciprocal: past any t at which the ray is still within 2^63 of the box, whose
-// squares are the last a float32 holds. At ordinary reciprocals it is nothing. (Farther out than
-// 1, where reciprocals are kept smaller, the roundings below are 2^102.)
-__device__ __forceinline__ float slabWidth(float3 id) {
-    const float least = fminf(fminf(fabsf(id.x), fabsf(id.y)), fabsf(id.z));
-    return least < kSlabReach ? least * 2.16840434e-19f : 0.f;  // 2^-62
-}
+// Terms of the slab distances from origin o. Where the reciprocal is clamped the distances are
+// not the ray's: they are moved by `reach` to either side, so that a box that the ray's line on
+// this axis lies in, or in whose plane it lies (0 times the reciprocal, where the difference
+// form's 0 inf drops the plane), is left out by no t. That widens boxes by reach / |id|: 2^-62
+// of the origin (or of 1) for a direction of length 1, 2^-23 for one of 2^-39.
 template <bool FUSED>
-__device__ __forceinline__ float slabNear(float o, float id, float width) {
+__device__ __forceinline__ float slabNear(float o, float id, float reach) {
     if constexpr (!FUSED) return o;
     const float q = o * id;  // infinite only with o, and then still so after the factor
-    return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -width * fabsf(id));
+    return fmaf(-q, q > 0.f ? 1.f + 3.f * kEps : 1.f - 3.f * kEps, -reach);
 }
 template <bool FUSED>
-__device__ __forceinline__ float slabFar(float o, float id, float width) {
+__device__ __forceinline__ float slabFar(float o, float id, float reach) {
     if constexpr (!FUSED) return o;
     const float q = o * id;
-    return fmaf(-q, q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps, width * fabsf(id));
+    return fmaf(-q, q > 0.f ? 1.f - 3.f * kEps : 1.f + 3.f * kEps, reach);
 }
 template <bool FUSED>
 __device__ __forceinline__ float slabAt(float p, float id, float c) {
     return FUSED ? fmaf(p, id, c) : (p - c) * id;
 }
 
-// Terms of L's slab distances for origins n of the near and f of the far planes (L.id set).
+// Terms of L's slab distances for origins n of the near and f of the far planes, the larger of
+// which bounded L.id's reciprocals. The reach of a ray is a t past any at which it can hit: 2^63
+// times its least reciprocal, where it is 2^63 from its origin (the last coordinates whose
+// squares a float32 holds), at most 2^125. Clamped on every axis it has no direction, or hits
+// beyond that; 2^101 is a unit in the last place of its origin then.
 template <bool FUSED>
 __device__ __forceinline__ void setSlabs(Level& L, float3 n, float3 f) {
-    const float w = FUSED ? slabWidth(L.id) : 0.f;
-    L.cn = make_float3(slabNear<FUSED>(n.x, L.id.x, w), slabNear<FUSED>(n.y, L.id.y, w), slabNear<FUSED>(n.z, L.id.z, w));
-    L.cf = make_float3(slabFar<FUSED>(f.x, L.id.x, w), slabFar<FUSED>(f.y, L.id.y, w), slabFar<FUSED>(f.z, L.id.z, w));
+    float3 w = make_float3(0.f, 0.f, 0.f);
+    if constexpr (FUSED) {
+        const float3 r = abs3(L.id);
+        const bool x = r.x >= slabCap(fmaxf(fabsf(n.x), fabsf(f.x))), y = r.y >= slabCap(fmaxf(fabsf(n.y), fabsf(f.y))),
+                   z = r.z >= slabCap(fmaxf(fabsf(n.z), fabsf(f.z)));
+        const float least = fminf(fminf(r.x, r.y), r.z);
+        const float reach = x && y && z ? 2.5353012e30f : fminf(least * 9.2233720e18f, 4.2535296e37f);
+        w = make_float3(x ? reach : 0.f, y ? reach : 0.f, z ? reach : 0.f);
+    }
+    L.cn = make_float3(slabNear<FUSED>(n.x, L.id.x, w.x), slabNear<FUSED>(n.y, L.id.y, w.y), slabNear<FUSED>(n.z, L.id.z, w.z));
+    L.cf = make_float3(slabFar<FUSED>(f.x, L.id.x, w.x), slabFar<FUSED>(f.y, L.id.y, w.y), slabFar<FUSED>(f.z, L.id.z, w.z));
 }
 
 template <bool FUSED>

@@ -1,7 +1,7 @@
 """Rays with zero direction components far from the origin of coordinates, where the product
 of the origin and a reciprocal direction leaves the range of a float32 (from 2^22 on at a
-reciprocal of 2^106), compared with the oracle; and rays in the planes of boxes whatever the
-length of their direction."""
+reciprocal of 2^106), compared with the oracle; rays in the planes of boxes whatever the
+length of their direction; and the work of rays with short directions."""
 import ctypes
 
 import numpy as np
@@ -123,7 +123,8 @@ def test_far_axis_aligned_rays_in_a_batch_and_a_user_kernel(gpu, user_lib, shift
 
 @pytest.mark.parametrize("fmt", list(FORMATS))
 @pytest.mark.parametrize("two_level", [False, True])
-@pytest.mark.parametrize("length, height", [(1.0, 1e9), (1e-4, 1.0), (1e-8, 1e4), (1e-12, 1.0), (1e-12, 1e8), (1e-20, 1e3)])
+@pytest.mark.parametrize("length, height", [(1.0, 1e9), (1e-4, 1.0), (1e-8, 1e4), (1e-12, 1.0), (1e-12, 1e8), (1e-20, 1e3),
+                                            (1e-30, 1.0)])
 def test_rays_in_box_planes_hit_with_directions_of_any_length(gpu, two_level, fmt, length, height):
     """Straight down on the vertices and edges of a flat grid in [-2, 0]^2: boxes have planes at 0,
     in which rays lie; edges belong to their triangles."""
@@ -149,6 +150,49 @@ def test_rays_in_box_planes_hit_with_directions_of_any_length(gpu, two_level, fm
     for any_hit in (False, True):
         got = _trace(gpu, r, any_hit=any_hit, **args)
         assert (got[1] != NONE).all() and np.all(np.abs(got[2] - t) <= 1e-5 * t)
+    if scene:
+        scene.close()
+    g.close()
+
+
+@pytest.mark.parametrize("fmt", list(FORMATS))
+@pytest.mark.parametrize("two_level", [False, True])
+@pytest.mark.parametrize("any_hit", [False, True])
+def test_short_and_zero_directions_are_culled(gpu, fmt, two_level, any_hit):
+    """Rays along an axis visit the same nodes whatever the length of their direction (to 2^-39 of
+    the mesh in width), rays without one in a geometry those around their origins."""
+    m = scenegen.terrain(64, 0.2)
+    g = Geometry(gpu, vertices=device_tensor(m.vertices), indices=device_tensor(m.indices), build_flags=FORMATS[fmt]).build()
+    scene = None
+    if two_level:
+        f = np.array([[0, 0, 0, 1, 1, 1, 1, 0, 0, 0]], np.float32)
+        scene = Scene(gpu, [g.handle], device_tensor(f), build_flags=FORMATS[fmt] if fmt == "wide8" else 0).build()
+    args = (scene.handle, None) if scene else (None, g.handle)
+    n = 4000
+    rng = np.random.default_rng(3)
+    rays = np.zeros((n, 8), np.float32)
+    rays[:, :3] = rng.uniform(-0.99, 0.99, (n, 3)) * [1, 0, 1] + [0, 1, 0]
+    rays[:, 7] = np.inf
+    hits = new_hits(n)
+
+    def nodes(length):
+        rays[:, 5] = -length
+        grt.grtGetTraceStatistics(gpu.handle)  # reads and clears
+        f = grt.grtTraceAnyHit if any_hit else grt.grtTraceClosest
+        f(gpu.handle, *args, device_tensor(rays), n, hits, None, grt.trace_options(flags=grt.GRT_TRACE_FLAG_COUNT))
+        found = (hits_to_numpy(hits)[1] != NONE).sum()
+        return grt.grtGetTraceStatistics(gpu.handle)["nodesVisited"] / n, found
+
+    want, all_hit = nodes(1.0)
+    assert all_hit == n
+    for length in (1e-6, 1e-9, 1e-12):
+        visited, found = nodes(length)
+        assert found == n and visited <= 1.1 * want, (length, visited, want)
+    if not two_level:  # an instance's boxes are widened without end for a ray that never leaves them
+        rays[:, 1] = 0.0  # among the triangles
+        visited, found = nodes(0.0)
+        assert found == 0 and visited <= 4 * want, (visited, want)
+    assert grt.grtGetLastDeviceError(gpu.handle) == grt.GRT_SUCCESS
     if scene:
         scene.close()
     g.close()
