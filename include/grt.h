@@ -368,7 +368,9 @@ typedef struct grtTraceOptions {
                                   grtTraceAmbientOcclusion, else 0.5) */
     uint32_t flags;            /* GRT_TRACE_FLAG_COUNT: accumulate grtTraceStatistics (slower) */
     void* globalStack;         /* optional caller-owned device buffer for the global entries; NULL = the
-                                  context's own (then traces on one context must not overlap in time) */
+                                  context's own (then traces on one context must not overlap in time).
+                                  With their own buffers at most 256 traces of a context may be in flight;
+                                  its last 1,024 captured ones share nothing with them or each other */
     size_t globalStackBytes;   /* size of globalStack; must be >= grtGetTraceGlobalStackSize */
     uint32_t rayMask;          /* ray mask (Sec. 7.5), ANDed with each instance's mask; 0 = all bits set */
 } grtTraceOptions;

@@ -209,8 +209,8 @@ __device__ __forceinline__ float slabAt(float p, float id, float c) {
 // Terms of L's slab distances for origins n of the near and f of the far planes, the larger of
 // which bounded L.id's reciprocals. The reach of a ray is a t past any at which it can hit: 2^63
 // times its least reciprocal, where it is 2^63 from its origin (the last coordinates whose
-// squares a float32 holds), at most 2^125. Clamped on every axis it has no direction, or hits
-// beyond that; 2^101 is a unit in the last place of its origin then.
+// squares a float32 holds), at most 2^125. Without a direction it hits nothing, and 2^101 is a
+// unit in the last place of its origin.
 template <bool FUSED>
 __device__ __forceinline__ void setSlabs(Level& L, float3 n, float3 f) {
     float3 w = make_float3(0.f, 0.f, 0.f);
@@ -219,7 +219,7 @@ __device__ __forceinline__ void setSlabs(Level& L, float3 n, float3 f) {
         const bool x = r.x >= slabCap(fmaxf(fabsf(n.x), fabsf(f.x))), y = r.y >= slabCap(fmaxf(fabsf(n.y), fabsf(f.y))),
                    z = r.z >= slabCap(fmaxf(fabsf(n.z), fabsf(f.z)));
         const float least = fminf(fminf(r.x, r.y), r.z);
-        const float reach = x && y && z ? 2.5353012e30f : fminf(least * 9.2233720e18f, 4.2535296e37f);
+        const float reach = norm1(L.d) == 0.f ? 2.5353012e30f : fminf(least * 9.2233720e18f, 4.2535296e37f);
         w = make_float3(x ? reach : 0.f, y ? reach : 0.f, z ? reach : 0.f);
     }
     L.cn = make_float3(slabNear<FUSED>(n.x, L.id.x, w.x), slabNear<FUSED>(n.y, L.id.y, w.y), slabNear<FUSED>(n.z, L.id.z, w.z));
